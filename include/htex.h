@@ -445,7 +445,7 @@ htex_status htex_rasterize_aniso(const htex_geometry* g, const float* view_proj,
  * channel 'channel' of the level-0 lookup at (h, u, v).
  *   t     textures of the same mesh;  tess  T in [1, 64]
  *   out   device [H][(T+1)(T+2)/2][3] float
- * Asynchronous; scratch as htex_rasterize. */
+ * Asynchronous; takes no scratch. */
 htex_status htex_displace(const htex_geometry* g, const htex_textures* t, int32_t tess, float scale,
                           int32_t channel, float* out, htex_stream stream);
 

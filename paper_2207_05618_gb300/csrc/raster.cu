@@ -1,8 +1,8 @@
-// The rendering side of Htex (paper Sections 3.1, 4.4, 5.1) as CUDA
-// kernels: Alg. 1 (the intrinsic triangle of each halfedge), rendering
-// the intrinsic triangulation into a per-pixel query buffer (halfedge,
-// perspective-correct barycentrics, footprint), and displacement of a
-// tessellated lattice along the input mesh's normals.
+// The rendering side of Htex (paper Sections 3.1, 4.4) as CUDA kernels:
+// Alg. 1 (the intrinsic triangle of each halfedge, evaluated once when the
+// geometry is made) and rendering the intrinsic triangulation into a
+// per-pixel query buffer (halfedge, perspective-correct barycentrics,
+// footprint).
 //
 // Rasterisation: one thread per intrinsic triangle covers the pixel
 // centres inside it (barycentrics >= 0, depth z/w in [-1, 1]) and keeps,
@@ -23,17 +23,8 @@
 
 #include <cuda_runtime.h>
 
+#include "geometry.h"
 #include "htex_internal.h"
-
-struct htex_geometry {
-    int32_t H = 0, V = 0, F = 0;
-    int32_t* d_next = nullptr;
-    int32_t* d_vert = nullptr;
-    int32_t* d_face = nullptr;
-    float* d_pos = nullptr;      // [V][3]
-    float* d_vn = nullptr;       // [V][3] vertex normals
-    float* d_fn = nullptr;       // [F][3] face normals
-};
 
 namespace {
 
@@ -43,29 +34,52 @@ __device__ __forceinline__ float3 ld3(const float* p, int32_t i) {
     return make_float3(p[3 * i], p[3 * i + 1], p[3 * i + 2]);
 }
 
+// What Alg. 1 reads; needed only while the geometry is made.
+struct Operators {
+    int32_t H;
+    const int32_t* next;
+    const int32_t* vert;
+    const int32_t* face;
+    const float* pos;   // [V][3]
+};
+
 // Alg. 1: v0 = Vert(Next h), v1 = the mean of the face's vertices walking
 // the Next cycle from h, v2 = Vert(h).
-__device__ __forceinline__ void alg1(const htex_geometry g, int32_t h, float3& v0, float3& v1, float3& v2) {
-    const int32_t nx = g.d_next[h];
-    v2 = ld3(g.d_pos, g.d_vert[h]);
-    v0 = ld3(g.d_pos, g.d_vert[nx]);
-    float3 c = v2;
-    int n = 1;
-    for (int32_t k = nx; k != h && n <= g.H; k = g.d_next[k]) {
-        const float3 p = ld3(g.d_pos, g.d_vert[k]);
-        c.x += p.x;
-        c.y += p.y;
-        c.z += p.z;
-        ++n;
+__global__ void k_alg1(Operators g, float4* tri) {
+    for (int32_t h = blockIdx.x * blockDim.x + threadIdx.x; h < g.H; h += gridDim.x * blockDim.x) {
+        const int32_t nx = g.next[h];
+        const float3 v2 = ld3(g.pos, g.vert[h]);
+        const float3 v0 = ld3(g.pos, g.vert[nx]);
+        float3 c = v2;
+        int n = 1;
+        for (int32_t k = nx; k != h && n <= g.H; k = g.next[k]) {
+            const float3 p = ld3(g.pos, g.vert[k]);
+            c.x += p.x;
+            c.y += p.y;
+            c.z += p.z;
+            ++n;
+        }
+        const float inv = 1.0f / float(n);
+        float4* t = tri + 3 * int64_t(h);
+        t[0] = make_float4(v0.x, v0.y, v0.z, __int_as_float(g.vert[nx]));
+        t[1] = make_float4(c.x * inv, c.y * inv, c.z * inv, __int_as_float(g.face[h]));
+        t[2] = make_float4(v2.x, v2.y, v2.z, __int_as_float(g.vert[h]));
     }
-    const float inv = 1.0f / float(n);
-    v1 = make_float3(c.x * inv, c.y * inv, c.z * inv);
+}
+
+// The intrinsic triangle of halfedge h.
+__device__ __forceinline__ void triangle(const htex_geometry& g, int32_t h, float3& v0, float3& v1, float3& v2) {
+    const float4* t = g.d_tri + 3 * int64_t(h);
+    const float4 a = __ldg(t), b = __ldg(t + 1), c = __ldg(t + 2);
+    v0 = make_float3(a.x, a.y, a.z);
+    v1 = make_float3(b.x, b.y, b.z);
+    v2 = make_float3(c.x, c.y, c.z);
 }
 
 __global__ void k_triangles(htex_geometry g, float* out) {
     for (int32_t h = blockIdx.x * blockDim.x + threadIdx.x; h < g.H; h += gridDim.x * blockDim.x) {
         float3 v0, v1, v2;
-        alg1(g, h, v0, v1, v2);
+        triangle(g, h, v0, v1, v2);
         float* o = out + 9 * int64_t(h);
         o[0] = v0.x; o[1] = v0.y; o[2] = v0.z;
         o[3] = v1.x; o[4] = v1.y; o[5] = v1.z;
@@ -130,7 +144,7 @@ __global__ void k_clear(unsigned long long* vis, int64_t n) {
 __global__ void k_raster(htex_geometry g, Camera cam, unsigned long long* vis) {
     for (int32_t h = blockIdx.x * blockDim.x + threadIdx.x; h < g.H; h += gridDim.x * blockDim.x) {
         float3 v[3];
-        alg1(g, h, v[0], v[1], v[2]);
+        triangle(g, h, v[0], v[1], v[2]);
         Screen s;
         if (!project(cam, v, s)) continue;
         const float xmin = fminf(s.x[0], fminf(s.x[1], s.x[2])), xmax = fmaxf(s.x[0], fmaxf(s.x[1], s.x[2]));
@@ -165,7 +179,7 @@ __global__ void k_resolve(htex_geometry g, Camera cam, const unsigned long long*
         if (key != ~0ull) {
             h = int32_t(uint32_t(key & 0xffffffffull));
             float3 v[3];
-            alg1(g, h, v[0], v[1], v[2]);
+            triangle(g, h, v[0], v[1], v[2]);
             Screen s;
             project(cam, v, s);
             const float px = float(i % cam.W) + 0.5f, py = float(i / cam.W) + 0.5f;
@@ -187,48 +201,6 @@ __global__ void k_resolve(htex_geometry g, Camera cam, const unsigned long long*
     }
 }
 
-// Displacement: lattice vertex k = (i, j), u = i/T, v = j/T of every
-// halfedge triangle; queries first, then positions from the lookups.
-__device__ __forceinline__ void lattice(int32_t k, int32_t T, float& u, float& v) {
-    // k enumerates i = 0..T, j = 0..T-i in order
-    int32_t i = 0, base = 0;
-    while (base + (T + 1 - i) <= k) {
-        base += T + 1 - i;
-        ++i;
-    }
-    u = float(i) / float(T);
-    v = float(k - base) / float(T);
-}
-
-__global__ void k_tess_queries(int32_t H, int32_t T, int32_t K, htex_query* q) {
-    const int64_t n = int64_t(H) * K;
-    for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < n; t += int64_t(gridDim.x) * blockDim.x) {
-        float u, v;
-        lattice(int32_t(t % K), T, u, v);
-        q[t] = htex_query{int32_t(t / K), u, v, 0.0f};
-    }
-}
-
-__global__ void k_displace(htex_geometry g, int32_t T, int32_t K, const float* d, int32_t C, int32_t channel,
-                           float scale, float* out) {
-    const int64_t n = int64_t(g.H) * K;
-    for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < n; t += int64_t(gridDim.x) * blockDim.x) {
-        const int32_t h = int32_t(t / K);
-        float u, v;
-        lattice(int32_t(t % K), T, u, v);
-        const float w = 1.0f - u - v;
-        float3 v0, v1, v2;
-        alg1(g, h, v0, v1, v2);
-        const float3 n2 = ld3(g.d_vn, g.d_vert[h]), n0 = ld3(g.d_vn, g.d_vert[g.d_next[h]]), n1 = ld3(g.d_fn, g.d_face[h]);
-        float3 N = make_float3(u * n2.x + v * n0.x + w * n1.x, u * n2.y + v * n0.y + w * n1.y, u * n2.z + v * n0.z + w * n1.z);
-        const float l = rsqrtf(N.x * N.x + N.y * N.y + N.z * N.z);
-        const float s = scale * d[t * C + channel] * l;
-        out[3 * t + 0] = u * v2.x + v * v0.x + w * v1.x + s * N.x;
-        out[3 * t + 1] = u * v2.y + v * v0.y + w * v1.y + s * N.y;
-        out[3 * t + 2] = u * v2.z + v * v0.z + w * v1.z + s * N.z;
-    }
-}
-
 int grid_for(int64_t n) {
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
@@ -238,10 +210,7 @@ int grid_for(int64_t n) {
 
 void free_geometry(htex_geometry* g) {
     if (!g) return;
-    cudaFree(g->d_next);
-    cudaFree(g->d_vert);
-    cudaFree(g->d_face);
-    cudaFree(g->d_pos);
+    cudaFree(g->d_tri);
     cudaFree(g->d_vn);
     cudaFree(g->d_fn);
     delete g;
@@ -301,19 +270,26 @@ extern "C" htex_status htex_geometry_create(const htex_mesh* m, const float* pos
     g->V = V;
     g->F = F;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    const size_t hb = sizeof(int32_t) * size_t(H);
-    bool ok = cudaMalloc(&g->d_next, hb) == cudaSuccess && cudaMalloc(&g->d_vert, hb) == cudaSuccess &&
-              cudaMalloc(&g->d_face, hb) == cudaSuccess &&
-              cudaMalloc(&g->d_pos, sizeof(float) * 3 * size_t(V)) == cudaSuccess &&
-              cudaMalloc(&g->d_vn, sizeof(float) * 3 * size_t(V)) == cudaSuccess &&
+    const size_t hb = sizeof(int32_t) * size_t(H), vb = sizeof(float) * 3 * size_t(V);
+    int32_t *next = nullptr, *vert = nullptr, *face = nullptr;
+    float* pos = nullptr;
+    bool ok = cudaMalloc(&next, hb) == cudaSuccess && cudaMalloc(&vert, hb) == cudaSuccess &&
+              cudaMalloc(&face, hb) == cudaSuccess && cudaMalloc(&pos, vb) == cudaSuccess &&
+              cudaMalloc(&g->d_tri, sizeof(float4) * 3 * size_t(H)) == cudaSuccess &&
+              cudaMalloc(&g->d_vn, vb) == cudaSuccess &&
               cudaMalloc(&g->d_fn, sizeof(float) * 3 * size_t(F)) == cudaSuccess;
-    ok = ok && cudaMemcpyAsync(g->d_next, m->next.data(), hb, cudaMemcpyHostToDevice, s) == cudaSuccess &&
-         cudaMemcpyAsync(g->d_vert, m->vert.data(), hb, cudaMemcpyHostToDevice, s) == cudaSuccess &&
-         cudaMemcpyAsync(g->d_face, m->face.data(), hb, cudaMemcpyHostToDevice, s) == cudaSuccess &&
-         cudaMemcpyAsync(g->d_pos, positions, sizeof(float) * 3 * size_t(V), cudaMemcpyHostToDevice, s) == cudaSuccess &&
-         cudaMemcpyAsync(g->d_vn, vn.data(), sizeof(float) * 3 * size_t(V), cudaMemcpyHostToDevice, s) == cudaSuccess &&
-         cudaMemcpyAsync(g->d_fn, fn.data(), sizeof(float) * 3 * size_t(F), cudaMemcpyHostToDevice, s) == cudaSuccess &&
-         cudaStreamSynchronize(s) == cudaSuccess;
+    ok = ok && cudaMemcpyAsync(next, m->next.data(), hb, cudaMemcpyHostToDevice, s) == cudaSuccess &&
+         cudaMemcpyAsync(vert, m->vert.data(), hb, cudaMemcpyHostToDevice, s) == cudaSuccess &&
+         cudaMemcpyAsync(face, m->face.data(), hb, cudaMemcpyHostToDevice, s) == cudaSuccess &&
+         cudaMemcpyAsync(pos, positions, vb, cudaMemcpyHostToDevice, s) == cudaSuccess &&
+         cudaMemcpyAsync(g->d_vn, vn.data(), vb, cudaMemcpyHostToDevice, s) == cudaSuccess &&
+         cudaMemcpyAsync(g->d_fn, fn.data(), sizeof(float) * 3 * size_t(F), cudaMemcpyHostToDevice, s) == cudaSuccess;
+    if (ok) k_alg1<<<grid_for(H), kThreads, 0, s>>>(Operators{H, next, vert, face, pos}, g->d_tri);
+    ok = ok && cudaGetLastError() == cudaSuccess && cudaStreamSynchronize(s) == cudaSuccess;
+    cudaFree(next);
+    cudaFree(vert);
+    cudaFree(face);
+    cudaFree(pos);
     if (!ok) {
         cudaGetLastError();
         free_geometry(g);
@@ -374,35 +350,4 @@ extern "C" htex_status htex_rasterize_aniso(const htex_geometry* g, const float*
                                             int32_t height, htex_query_aniso* queries, float* depth,
                                             htex_stream stream) {
     return rasterize(g, view_proj, width, height, queries, depth, stream);
-}
-
-extern "C" htex_status htex_displace(const htex_geometry* g, const htex_textures* t, int32_t tess, float scale,
-                                     int32_t channel, float* out, htex_stream stream) {
-    if (!g || !t || !out || tess < 1 || tess > 64 || channel < 0 || channel >= t->C || t->H != g->H)
-        return HTEX_ERR_INVALID_ARG;
-    const int32_t K = (tess + 1) * (tess + 2) / 2;
-    const int64_t n = int64_t(g->H) * K;
-    if (n >= (int64_t(1) << 31)) return HTEX_ERR_INVALID_ARG;
-    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return HTEX_ERR_CUDA;
-    cudaMemPool_t pool = work_pool(dev);
-    if (!pool) return HTEX_ERR_CUDA;
-    void* work = nullptr;
-    const size_t qb = size_t(n) * sizeof(htex_query), db = size_t(n) * sizeof(float) * size_t(t->C);
-    if (cudaMallocFromPoolAsync(&work, qb + db, pool, s) != cudaSuccess) {
-        cudaGetLastError();
-        return HTEX_ERR_OUT_OF_MEMORY;
-    }
-    auto* q = static_cast<htex_query*>(work);
-    auto* d = reinterpret_cast<float*>(static_cast<uint8_t*>(work) + qb);
-    k_tess_queries<<<grid_for(n), kThreads, 0, s>>>(g->H, tess, K, q);
-    htex_status st = cudaGetLastError() == cudaSuccess ? HTEX_OK : HTEX_ERR_CUDA;
-    if (st == HTEX_OK) st = htex_launch_lookup(t, q, n, d, HTEX_LOOKUP_GLOBAL, stream, nullptr);
-    if (st == HTEX_OK) {
-        k_displace<<<grid_for(n), kThreads, 0, s>>>(*g, tess, K, d, t->C, channel, scale, out);
-        if (cudaGetLastError() != cudaSuccess) st = HTEX_ERR_CUDA;
-    }
-    cudaFreeAsync(work, s);
-    return st;
 }

@@ -136,3 +136,24 @@ def test_displacement_matches_oracle_and_is_crack_free():
     for grp in np.unique(inv):
         pts = flat[inv == grp]
         assert np.abs(pts - pts[0]).max() < 2e-5
+
+
+@pytest.mark.parametrize("dtype,C,channel", [("f32", 3, 2), ("u8", 4, 0), ("u8", 3, 1), ("f16", 1, 0), ("bf16", 2, 1),
+                                             ("e4m3", 4, 3)])
+@pytest.mark.parametrize("T", [1, 2, 3, 8, 64])
+def test_displacement_formats_and_block_edges(dtype, C, channel, T):
+    """Mixed resolutions down to 1x1, every texel format, and the halfedges
+    per block at both ends (T = 1: 256 with a partial last block; T = 64: 1).
+    Tolerance: the FP32 lookup's 1e-5 and the position's few ulp, as above."""
+    fs, fv, V, pos = syn.cylinder(around=16, rows=6, seed=4)
+    mo = oracle.mesh_from_faces(fs, fv, V)
+    mesh = hx.Mesh(fs, fv, V)
+    assert mesh.H % 256 != 0 and mesh.H > 256
+    log2n = np.random.default_rng(1).integers(0, 6, mesh.E).astype(np.int32)
+    flags = hx.BUILD_MIPS | hx.MIRROR_BOUNDARY
+    texels = (syn.texels_u8 if dtype == "u8" else syn.texels_f32)(log2n, C, 3)
+    tl = hx.Textures.upload(mesh, log2n, texels, C, dtype, flags)
+    to = oracle.prepare_textures(mo, log2n, texels, C, dtype, flags)
+    got = render.Geometry(mesh, pos).displace(tl, T, 0.3, channel=channel).cpu().numpy()
+    pos32 = pos.astype(np.float32).astype(np.float64)
+    np.testing.assert_allclose(got, oracle.displace(mo, to, pos32, T, 0.3, channel=channel), atol=2e-5)
