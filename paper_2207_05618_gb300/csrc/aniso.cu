@@ -18,18 +18,18 @@
 //     Alg. 2, with full 2x2 zero-bordered taps (a probe off the triangle can
 //     reach any texel of the neighbouring quads); the result is the summed
 //     data over the summed normalisation weight.
-// Work distribution: a warp takes 32 queries at a time and works through
-// all of their probes together, 32 (query, probe) pairs per round, so a
-// warp whose lanes need 1 to 16 probes runs ceil(sum K / 32) rounds instead
-// of its largest K.  Each query's constants (centre, scaled major axis, K,
-// and for each fetch its two levels' offsets, sizes and weights, code
-// factor and reflection) are computed once by its own lane and kept in
-// shared memory for the lanes that run its probes; each round's probe
-// results (data and weight sums) go through shared memory back to the
-// lanes of their queries, which add them in probe order, so that a query's
-// result does not depend on which other queries share its warp.  A fetch whose
-// quad no probe of the round can reach (more than half a coarsest-level
-// texel outside it) is skipped warp-uniformly.
+// Work distribution: a warp takes 32 queries and works through their items
+// -- one (fetch, probe) pair whose probe can reach the fetch's quad, both
+// levels -- 32 at a time, in the order of query, fetch, probe, so that
+// neighbouring lanes read neighbouring texels.  Which probes reach a fetch
+// is an interval of probe numbers (the probes lie on a line and the reach is
+// a box), so the items are counted without visiting the probes.  Each
+// query's constants are computed once by its own lane and kept in shared
+// memory; each round's item sums go through shared memory to lanes that add
+// them to their query's, one lane per query and channel, in item order: a
+// query's result does not depend on which other queries share its warp.
+#include <algorithm>
+
 #include <cuda_runtime.h>
 
 #include "lookup_core.cuh"
@@ -60,68 +60,71 @@ __device__ __forceinline__ TapsG taps_g(float p, int N) {
     return TapsG{i, (i >= 0 && i < N) ? 1.0f - a : 0.0f, (i + 1 >= 0 && i + 1 < N) ? a : 0.0f};
 }
 
-// Per-query constants of one fetch, fixed over its probes: where its two
-// levels start, their sizes and weights, the code factor and the Alg. 2
-// reflection.
-struct FetchConst {
-    int64_t base0;          // byte offset of texel (0, 0) of level l0
-    int32_t d1;             // byte offset of level l1 from level l0 (0 when one level is read)
-    int16_t n0, n1;         // log2 of their sizes (l1 = l0 when one level is read)
-    float w0, w1;           // their weights (w1 = 0 when one level is read)
-    float sc;               // code factor
-    uint32_t flip;          // Alg. 2 reflection
+// One level of one fetch at quad coordinates (x, y): four taps, their data
+// weights (level weight and code scale included) and their loads.
+template <int DT, int C>
+struct LevelTaps {
+    static constexpr int TB = C * Fmt<DT>::ES;
+    uint64_t o;
+    uint32_t row;
+    float w[4];
+
+    // wl: the level weight; wd: the level weight times the code scale.
+    // Returns the level's share of the normalisation weight.
+    __device__ __forceinline__ float plan(uint64_t base, int n, float x, float y, float wl, float wd) {
+        const int N = 1 << n;
+        const TapsG tx = taps_g(x, N), ty = taps_g(y, N);
+        const float y0 = ty.w0 * wd, y1 = ty.w1 * wd;
+        w[0] = y0 * tx.w0;
+        w[1] = y0 * tx.w1;
+        w[2] = y1 * tx.w0;
+        w[3] = y1 * tx.w1;
+        o = base + uint64_t(int64_t(((ty.i << n) + tx.i) * TB));
+        row = uint32_t(TB) << n;
+        return wl * (tx.w0 + tx.w1) * (ty.w0 + ty.w1);
+    }
+    __device__ __forceinline__ uint64_t at(int k) const { return o + (k & 1 ? TB : 0) + (k & 2 ? row : 0u); }
 };
 
-template <int DT, int C>
-__device__ __forceinline__ FetchConst fetch_const(const TexRef& t, const Lod& d, uint32_t code) {
-    constexpr int TB = C * Fmt<DT>::ES;
-    FetchConst f;
-    const int l1 = d.l1 >= 0 ? d.l1 : d.l0;
-    f.n0 = int16_t(t.n - d.l0);
-    f.n1 = int16_t(t.n - l1);
-    f.base0 = int64_t(t.off) + int64_t(level_texels(t.n, d.l0)) * TB;
-    f.d1 = int32_t(int64_t(level_texels(t.n, l1) - level_texels(t.n, d.l0)) * TB);
-    f.w0 = d.w0;
-    f.w1 = d.l1 >= 0 ? d.w1 : 0.0f;
-    f.sc = code_factor<DT>(t);
-    f.flip = code & kFlipBit;
-    return f;
+// Shared-memory words of a query: centre u, v, the probe spacing axis (major
+// axis times s) mu, mv, K and 1 / (2K); then for each fetch with items
+// (own, Next, Prev, those without left out) the byte offset of texel (0, 0)
+// of its finer level (low and high half), the packed fields below, the
+// coarser level's weight and, for the scaled formats, the code scale.
+enum { kU, kV, kMu, kMv, kK, kInv2K, kFetch };
+// packed: log2 sizes of the two levels (4 bits each), first probe (4), then:
+// one level only, coordinates swapped, x negated, y negated, x and y offset
+// by one (Alg. 2's reflection)
+constexpr uint32_t kOneLevel = 1u << 12, kSwap = 1u << 13, kNegX = 1u << 14, kNegY = 1u << 15, kOffset = 1u << 16;
+
+// The probes k = 0..K-1, at t = (2k + 1 - K) / (2K), for which lo < c + m t
+// < hi, as an interval [k0, k1); it may hold a probe too many at either end
+// (whose taps all have weight zero), never one too few.
+__device__ __forceinline__ void cut_probes(float c, float inv_m, float lo, float hi, float Kf, float& k0, float& k1) {
+    // inv_m = +-inf: m = 0 (or so small that every probe sits at c): the
+    // bounds come out infinite, or NaN on the border, which min and max drop
+    const float a = (lo - c) * inv_m, b = (hi - c) * inv_m;
+    const float shift = 0.5f * Kf - 0.5f;
+    k0 = fmaxf(k0, fmaf(fminf(a, b), Kf, shift) - 0.01f);
+    k1 = fminf(k1, fmaf(fmaxf(a, b), Kf, shift) + 0.01f);
 }
 
-// One level of one fetch at quad coordinates (x, y) with level weight wl.
-template <int DT, int C>
-__device__ __forceinline__ void aniso_level(const Asset<GlobalSpace>& A, int64_t base, int N, float x, float y,
-                                            float wl, float sc, float (&acc)[C], float& W) {
-    constexpr int TB = C * Fmt<DT>::ES;
-    const TapsG tx = taps_g(x, N), ty = taps_g(y, N);
-    W += wl * (tx.w0 + tx.w1) * (ty.w0 + ty.w1);
-    const float y0 = ty.w0 * wl, y1 = ty.w1 * wl;
-    const float w[4] = {y0 * tx.w0, y0 * tx.w1, y1 * tx.w0, y1 * tx.w1};
-    const int64_t o = base + (int64_t(ty.i) * N + tx.i) * TB;
-    const int64_t d[4] = {0, TB, int64_t(N) * TB, int64_t(N) * TB + TB};
+// First probe and one past the last of the three fetches: the own quad
+// within h0 of [0, 1]^2, the Next quad (coordinates (v, -u)) within h1, the
+// Prev quad ((-v, u)) within h2 (half a texel of the coarser level each,
+// and 1e-6 for the coordinates' own rounding).
+__device__ __forceinline__ void probe_ranges(float u, float v, float mu, float mv, int K, const float (&half)[3],
+                                             int (&first)[3], int (&last)[3]) {
+    const float iu = __frcp_rn(mu), iv = __frcp_rn(mv), Kf = float(K);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        float v[C];
-        load_texel_if<DT, C>(A.pool, w[k] != 0.0f, uint64_t(o + d[k]), v);
-        const float wd = w[k] * sc;
-#pragma unroll
-        for (int c = 0; c < C; ++c) acc[c] = fmaf(wd, v[c], acc[c]);
+    for (int e = 0; e < 3; ++e) {
+        const float h = half[e] + 1e-6f;
+        float k0 = 0.0f, k1 = Kf - 1.0f;
+        cut_probes(u, iu, e == 1 ? -1.0f - h : -h, e == 1 ? h : 1.0f + h, Kf, k0, k1);
+        cut_probes(v, iv, e == 2 ? -1.0f - h : -h, e == 2 ? h : 1.0f + h, Kf, k0, k1);
+        first[e] = max(0, int(ceilf(k0)));
+        last[e] = max(first[e], min(K, int(floorf(k1)) + 1));
     }
-}
-
-// One fetch of one probe (one or two levels), skipped when no lane of the
-// warp has a tap in bounds.
-template <int DT, int C>
-__device__ __forceinline__ void aniso_fetch(const Asset<GlobalSpace>& A, bool on, const FetchConst& f, float a,
-                                            float b, float (&acc)[C], float& W) {
-    const float x = f.flip ? 1.0f - a : a, y = f.flip ? 1.0f - b : b;
-    const float half = __int_as_float((126 - f.n1) << 23);   // 2^-(n1 + 1): half a texel of the coarser level
-    const bool near = on && x > -half && x < 1.0f + half && y > -half && y < 1.0f + half;
-    if (!__any_sync(0xffffffffu, near)) return;
-    aniso_level<DT, C>(A, f.base0, 1 << f.n0, x, y, near ? f.w0 : 0.0f, f.sc, acc, W);
-    const bool two = near && f.w1 != 0.0f;
-    if (__any_sync(0xffffffffu, two))
-        aniso_level<DT, C>(A, f.base0 + f.d1, 1 << f.n1, x, y, two ? f.w1 : 0.0f, f.sc, acc, W);
 }
 
 // Probe count (see the file comment): same float operations as the oracle.
@@ -133,127 +136,241 @@ __device__ __forceinline__ int aniso_probes(float px2, float py2, int kmax) {
     return max(1, int(ceilf(r)));
 }
 
-// One block of 1024 threads per SM (156 KiB of per-warp shared state):
-// measured 7% faster than four blocks of 256 per SM on the asset-scale
-// anisotropic batch
-constexpr int kAnisoThreads = 1024;
+constexpr int kAnisoThreads = 128;
 constexpr int kAnisoWarps = kAnisoThreads / 32;
-constexpr int kAnisoMaxK = 16;
+// Resident blocks per SM (56 registers a thread).  The kernel is bound by
+// random 128-byte lines from DRAM and their latency: 4M queries of 1..16
+// probes on a 1.4 GB RGBA8 asset take 582 / 538 / 551 / 586 us at 8 / 9 /
+// 10 / 11 blocks (2.8 GB of lines, 5.2 TB/s at 9; independent random lines
+// reach 5.2 TB/s).
+constexpr int kAnisoBlocks = 9;
 
-// One query's constants, written by its lane, read by the lanes that run
-// its probes.  120 bytes (30 words), so that lanes reading the same field
-// of different queries hit different shared-memory banks (a size of 32
-// words put them all in one bank).
+// A decoded anisotropic query: validity, the probe count and line, and the
+// footprint of one probe.
 struct AnisoQuery {
-    float u, v, mu, mv;     // centre and the probe spacing axis (major axis times s)
-    int32_t K;              // probes (0: the lane holds no query)
-    float inv2K;            // +-1 / (2K), negative for an invalid query: probe k sits at t = (2k + 1 - K) / (2K)
-    FetchConst f[3];        // own, Next, Prev
+    bool ok;
+    int h, K;
+    float u, v, mu, mv, footprint;
 };
-static_assert(sizeof(AnisoQuery) == 120, "AnisoQuery: 30 words (bank spread)");
+
+__device__ __forceinline__ AnisoQuery decode_aniso(int4 r0, int4 r1, int32_t H, int kmax) {
+    AnisoQuery Q;
+    const float dudx = __int_as_float(r1.x), dvdx = __int_as_float(r1.y);
+    const float dudy = __int_as_float(r1.z), dvdy = __int_as_float(r1.w);
+    const float px2 = __fadd_rn(__fmul_rn(dudx, dudx), __fmul_rn(dvdx, dvdx));
+    const float py2 = __fadd_rn(__fmul_rn(dudy, dudy), __fmul_rn(dvdy, dvdy));
+    float f;
+    Q.ok = decode_query(make_int4(r0.x, r0.y, r0.z, 0), H, Q.h, Q.u, Q.v, f);
+    Q.ok = Q.ok && isfinite(dudx) && isfinite(dvdx) && isfinite(dudy) && isfinite(dvdy) && isfinite(px2) &&
+           isfinite(py2);
+    Q.K = Q.ok ? aniso_probes(px2, py2, kmax) : 0;
+    const bool major_y = py2 > px2;
+    const float pmax = sqrtf(fmaxf(px2, py2));
+    const float s = pmax > float(max(Q.K, 1)) ? float(Q.K) / pmax : 1.0f;
+    Q.mu = (major_y ? dudy : dudx) * s;
+    Q.mv = (major_y ? dvdy : dvdx) * s;
+    Q.footprint = Q.ok ? pmax / float(Q.K) : 0.0f;
+    return Q;
+}
 
 template <int DT, int C>
-__global__ void __launch_bounds__(kAnisoThreads) k_lookup_aniso(Asset<GlobalSpace> A, AnisoParams p) {
-    __shared__ AnisoQuery sq[kAnisoWarps][32];
-    __shared__ uint8_t owner[kAnisoWarps][32 * kAnisoMaxK];   // the query lane of each of the warp's probes
-    __shared__ float pr[kAnisoWarps][C + 1][32];             // one round's probe results: data and weight sums
+__global__ void __launch_bounds__(kAnisoThreads, kAnisoBlocks) k_lookup_aniso(Asset<GlobalSpace> A, AnisoParams p) {
+    constexpr int TB = C * Fmt<DT>::ES;
+    constexpr int FW = Fmt<DT>::SCALED ? 5 : 4;      // words per fetch
+    __shared__ uint32_t consts[kAnisoWarps][kFetch + 3 * FW][32];
+    constexpr int SW = (C + 1) | 1;                  // words of an item's sums, odd (bank spread)
+    __shared__ float part[kAnisoWarps][32][SW];      // one round's item sums: data and weight
+    __shared__ float total[kAnisoWarps][32][SW];     // the queries' sums
+    __shared__ uint8_t mark[kAnisoWarps][32];        // the fetch that starts at an item of the round
     const unsigned lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
-    const int64_t warps = int64_t(gridDim.x) * kAnisoWarps;
-    for (int64_t base = (int64_t(blockIdx.x) * kAnisoWarps + wib) * 32; base < p.n; base += warps * 32) {
-        // ---- this lane's query: decode, probe count, per-fetch constants
+    uint32_t (*const cw)[32] = consts[wib];
+    const htex_query* const qq = reinterpret_cast<const htex_query*>(p.q);   // two 16-byte words a query
+    const int64_t step = int64_t(gridDim.x) * kAnisoThreads;
+    for (int64_t base = int64_t(blockIdx.x) * kAnisoThreads + wib * 32; base < p.n; base += step) {
+        // ---- this lane's query: decode, probe count, the fetches with items
         const int64_t i = base + lane;
         const bool valid = i < p.n;
-        const int4 r0 = valid ? ld_query(reinterpret_cast<const htex_query*>(p.q), 2 * i) : make_int4(-1, 0, 0, 0);
-        const int4 r1 = valid ? ld_query(reinterpret_cast<const htex_query*>(p.q), 2 * i + 1) : make_int4(0, 0, 0, 0);
-        const float dudx = __int_as_float(r1.x), dvdx = __int_as_float(r1.y);
-        const float dudy = __int_as_float(r1.z), dvdy = __int_as_float(r1.w);
-        const float px2 = __fadd_rn(__fmul_rn(dudx, dudx), __fmul_rn(dvdx, dvdx));
-        const float py2 = __fadd_rn(__fmul_rn(dudy, dudy), __fmul_rn(dvdy, dvdy));
-        int h;
-        float u, v, f;
-        bool ok = valid && decode_query(make_int4(r0.x, r0.y, r0.z, 0), A.H, h, u, v, f);
-        ok = ok && isfinite(dudx) && isfinite(dvdx) && isfinite(dudy) && isfinite(dvdy) && isfinite(px2) &&
-             isfinite(py2);
-        if (!ok) {
-            u = 0.0f;
-            v = 0.0f;
-            if (valid && p.status) atomicAdd(p.status, 1);
-        }
-        const int K = valid ? (ok ? aniso_probes(px2, py2, p.kmax) : 1) : 0;
-        const bool major_y = py2 > px2;
-        const float pmax = sqrtf(fmaxf(px2, py2));
-        const float s = pmax > float(max(K, 1)) ? float(K) / pmax : 1.0f;
-        const float lf = footprint_log2(ok ? pmax / float(K) : 0.0f);
-        const uint4 rec = ok ? A.rec.ld16(uint64_t(h) * 16u) : make_uint4(0, 0, 0, 0);
-        const TexRef to = tex_ref<DT>(A, rec.x & ~kFlipBit);
-        const TexRef tn = tex_ref<DT>(A, rec.y & ~kFlipBit);
-        const TexRef tp = tex_ref<DT>(A, rec.z & ~kFlipBit);
-        AnisoQuery& Q = sq[wib][lane];
-        Q.u = u;
-        Q.v = v;
-        Q.mu = (major_y ? dudy : dudx) * s;
-        Q.mv = (major_y ? dvdy : dvdx) * s;
-        Q.K = K;
-        Q.inv2K = (ok ? 1.0f : -1.0f) / float(2 * max(K, 1));
-        Q.f[0] = fetch_const<DT, C>(to, select_lod(lf, to.n), rec.x);
-        Q.f[1] = fetch_const<DT, C>(tn, select_lod(lf, tn.n), rec.y);
-        Q.f[2] = fetch_const<DT, C>(tp, select_lod(lf, tp.n), rec.z);
-        float qacc[C];
+        const int4 r0 = valid ? ld_query(qq, 2 * i) : make_int4(-1, 0, 0, 0);
+        const int4 r1 = valid ? ld_query(qq, 2 * i + 1) : make_int4(0, 0, 0, 0);
+        const AnisoQuery Q = decode_aniso(r0, r1, A.H, p.kmax);
+        if (valid && !Q.ok && p.status) atomicAdd(p.status, 1);
+        int slots = 0, len[3] = {0, 0, 0};
+        if (Q.ok) {
+            const uint4 rec = A.rec.ld16(uint64_t(Q.h) * 16u);
+            const uint32_t code[3] = {rec.x, rec.y, rec.z};
+            const float lf = footprint_log2(Q.footprint);
+            TexRef t[3];
+            Lod d[3];
+            float half[3];
 #pragma unroll
-        for (int c = 0; c < C; ++c) qacc[c] = 0.0f;
-        float qW = 0.0f;
+            for (int e = 0; e < 3; ++e) {
+                t[e] = tex_ref<DT>(A, code[e] & ~kFlipBit);
+                d[e] = select_lod(lf, t[e].n);
+                half[e] = __int_as_float((126 - (t[e].n - coarsest(d[e]))) << 23);   // 2^-(log2 size + 1)
+            }
+            int first[3], last[3];
+            probe_ranges(Q.u, Q.v, Q.mu, Q.mv, Q.K, half, first, last);
+#pragma unroll
+            for (int e = 0; e < 3; ++e) {
+                if (last[e] <= first[e]) continue;
+                const bool flip = code[e] & kFlipBit, one = d[e].l1 < 0;
+                // own (u, v), Next (v, -u), Prev (-v, u), each (1 - x, 1 - y) when reflected
+                const uint32_t turn = (e ? kSwap : 0u) | ((e == 2) != flip ? kNegX : 0u) |
+                                      ((e == 1) != flip ? kNegY : 0u) | (flip ? kOffset : 0u);
+                const uint64_t o = t[e].off + uint64_t(level_texels(t[e].n, d[e].l0)) * TB;
+                uint32_t (*f)[32] = cw + kFetch + slots * FW;
+                f[0][lane] = uint32_t(o);
+                f[1][lane] = uint32_t(o >> 32);
+                f[2][lane] = uint32_t(t[e].n - d[e].l0) | uint32_t(t[e].n - coarsest(d[e])) << 4 |
+                             uint32_t(first[e]) << 8 | (one ? kOneLevel : 0u) | turn;
+                f[3][lane] = __float_as_uint(one ? 0.0f : d[e].w1);
+                if constexpr (Fmt<DT>::SCALED) f[4][lane] = __float_as_uint(t[e].scale);
+                const int l = last[e] - first[e];
+                if (slots == 0) len[0] = l;
+                else if (slots == 1) len[1] = l;
+                else len[2] = l;
+                ++slots;
+            }
+            cw[kU][lane] = __float_as_uint(Q.u);
+            cw[kV][lane] = __float_as_uint(Q.v);
+            cw[kMu][lane] = __float_as_uint(Q.mu);
+            cw[kMv][lane] = __float_as_uint(Q.mv);
+            cw[kK][lane] = uint32_t(Q.K);
+            cw[kInv2K][lane] = __float_as_uint(1.0f / float(2 * Q.K));
+        }
+#pragma unroll
+        for (int c = 0; c <= C; ++c) total[wib][lane][c] = 0.0f;
 
-        // ---- the warp's probes in order: query lane by lane, probe by probe
-        int incl = K;
+        // ---- the warp's items: where each query's fetches start
+        const int items = len[0] + len[1] + len[2];
+        int incl = items;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
             const int o = __shfl_up_sync(0xffffffffu, incl, d);
             if (lane >= unsigned(d)) incl += o;
         }
-        const int first = incl - K;                          // this lane's first probe
-        const int P = __shfl_sync(0xffffffffu, incl, 31);     // the warp's probes
-        for (int k = 0; k < K; ++k) owner[wib][first + k] = uint8_t(lane);
-        __syncwarp();
+        const int P = __shfl_sync(0xffffffffu, incl, 31);
+        const int start = incl - items;
+        const uint32_t span = uint32_t(start) | uint32_t(incl) << 16;   // this lane's query's items
+        uint32_t seg = 0;    // query and slot running on from the round before, and where it started
+        int seg_start = 0;
 
-        for (int r0p = 0; r0p < P; r0p += 32) {
-            const int j = r0p + int(lane);
-            const bool has = j < P;
-            const int q = has ? owner[wib][j] : int(owner[wib][P - 1]);
-            const int qfirst = __shfl_sync(0xffffffffu, first, q);
-            const AnisoQuery& R = sq[wib][q];
-            const bool on = has && R.inv2K > 0.0f;
-            const int KR = R.K, k = j - qfirst;
-            const float t = float(2 * k + 1 - KR) * R.inv2K;
-            const float pu = fmaf(R.mu, t, R.u), pv = fmaf(R.mv, t, R.v);
-            float acc[C];
+        for (int R = 0; R < P; R += 32) {
+            // each lane's item: mark where fetches start, look left for the nearest mark
+            uint32_t starts = 0;
+            int at = start - R;
 #pragma unroll
-            for (int c = 0; c < C; ++c) acc[c] = 0.0f;
-            float W = 0.0f;
-            aniso_fetch<DT, C>(A, on, R.f[0], pu, pv, acc, W);
-            aniso_fetch<DT, C>(A, on, R.f[1], pv, -pu, acc, W);
-            aniso_fetch<DT, C>(A, on, R.f[2], -pv, pu, acc, W);
-#pragma unroll
-            for (int c = 0; c < C; ++c) pr[wib][c][lane] = acc[c];
-            pr[wib][C][lane] = W;
-            __syncwarp();
-            // each lane adds the probes of its own query that this round
-            // computed, in probe order: the same sums whatever the other
-            // queries of the warp are
-            const int a = max(first, r0p) - r0p, b = min(first + K, r0p + 32) - r0p;
-            for (int m = a; m < b; ++m) {
-#pragma unroll
-                for (int c = 0; c < C; ++c) qacc[c] += pr[wib][c][m];
-                qW += pr[wib][C][m];
+            for (int s = 0; s < 3; ++s) {
+                if (len[s] > 0 && unsigned(at) < 32u) {
+                    mark[wib][at] = uint8_t(lane | unsigned(s) << 5);
+                    starts |= 1u << at;
+                }
+                at += len[s];
             }
+            starts = __reduce_or_sync(0xffffffffu, starts);
+            __syncwarp();
+            const uint32_t before = starts & (0xffffffffu >> (31u - lane));
+            if (before) {
+                const int m = 31 - __clz(int(before));
+                seg = mark[wib][m];
+                seg_start = R + m;
+            }
+            const int j = R + int(lane);
+            const bool has = j < P;
+            const unsigned q = seg & 31u;
+            uint32_t (*f)[32] = cw + kFetch + (seg >> 5) * FW;
+            const uint32_t c2 = f[2][q];
+            const uint64_t o0 = uint64_t(f[1][q]) << 32 | f[0][q];
+            const int n0 = int(c2 & 15u), n1 = int(c2 >> 4 & 15u);
+            const float w1 = has ? __uint_as_float(f[3][q]) : 0.0f, w0 = has ? 1.0f - w1 : 0.0f;
+            float scale = 1.0f;
+            if constexpr (Fmt<DT>::SCALED) scale = __uint_as_float(f[4][q]);
+            const int k = int(c2 >> 8 & 15u) + j - seg_start;
+            const float t = float(2 * k + 1 - int(cw[kK][q])) * __uint_as_float(cw[kInv2K][q]);
+            const float pu = fmaf(__uint_as_float(cw[kMu][q]), t, __uint_as_float(cw[kU][q]));
+            const float pv = fmaf(__uint_as_float(cw[kMv][q]), t, __uint_as_float(cw[kV][q]));
+            const bool swap = c2 & kSwap;
+            const float off = (c2 & kOffset) ? 1.0f : 0.0f;
+            const float a = swap ? pv : pu, b = swap ? pu : pv;
+            const float x = off + ((c2 & kNegX) ? -a : a), y = off + ((c2 & kNegY) ? -b : b);
+
+            Sums<C> acc;
+            LevelTaps<DT, C> L0, L1;
+            float W = L0.plan(o0, n0, x, y, w0, w0 * scale);
+            const bool two = __any_sync(0xffffffffu, w1 != 0.0f);
+            // the coarser level's texels follow the finer one's (its own when there is no coarser one)
+            const uint64_t o1 = o0 + (uint64_t(TB) << (2 * n0));
+            if constexpr (TB <= 8 && (TB & (TB - 1)) == 0 && (DT != HTEX_F32 || C == 1)) {
+                Raw<DT, C> ta[4], tb[4];   // every load before the first decode
+#pragma unroll
+                for (int m = 0; m < 4; ++m) ta[m].load_if(A.pool, L0.w[m] != 0.0f, L0.at(m), l2_leave_policy());
+                if (two) {
+                    W += L1.plan(o1, n1, x, y, w1, w1 * scale);
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) tb[m].load_if(A.pool, L1.w[m] != 0.0f, L1.at(m), l2_leave_policy());
+                }
+                float v[C];
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    ta[m].decode(v);
+                    acc.fma(L0.w[m], v);
+                }
+                if (two) {
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) {
+                        tb[m].decode(v);
+                        acc.fma(L1.w[m], v);
+                    }
+                }
+            } else {
+                float v[4][C];
+#pragma unroll
+                for (int m = 0; m < 4; ++m) load_texel_if<DT, C>(A.pool, L0.w[m] != 0.0f, L0.at(m), v[m]);
+#pragma unroll
+                for (int m = 0; m < 4; ++m) acc.fma(L0.w[m], v[m]);
+                if (two) {
+                    W += L1.plan(o1, n1, x, y, w1, w1 * scale);
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) load_texel_if<DT, C>(A.pool, L1.w[m] != 0.0f, L1.at(m), v[m]);
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) acc.fma(L1.w[m], v[m]);
+                }
+            }
+            float sums[C];
+            acc.get(sums);
+#pragma unroll
+            for (int c = 0; c < C; ++c) part[wib][lane][c] = sums[c];
+            part[wib][lane][C] = W;
+            __syncwarp();
+
+            // add them to their queries' sums: a lane per query and channel
+            // (data or weight), the items in order
+            const int end = min(P - R, 32);
+            const int q0 = __shfl_sync(0xffffffffu, int(q), 0), q1 = __shfl_sync(0xffffffffu, int(q), end - 1);
+            constexpr int PER = 32 / (C + 1);   // queries per pass
+            const int qr = int(lane) / (C + 1), ch = int(lane) - qr * (C + 1);
+            for (int qb = q0; qb <= q1; qb += PER) {
+                const int qi = qb + qr;
+                const uint32_t sp = __shfl_sync(0xffffffffu, span, qi & 31);
+                if (qr < PER && qi <= q1) {
+                    const int lo = max(int(sp & 0xffffu) - R, 0), hi = min(int(sp >> 16) - R, end);
+                    float s = total[wib][qi][ch];
+#pragma unroll 4
+                    for (int m = lo; m < hi; ++m) s += part[wib][m][ch];
+                    total[wib][qi][ch] = s;
+                }
+            }
+            seg = __shfl_sync(0xffffffffu, seg, 31);
+            seg_start = __shfl_sync(0xffffffffu, seg_start, 31);
             __syncwarp();
         }
 
         // ---- normalise and store (invalid queries: W = 0, data 0, 0 * inf = NaN)
         if (valid) {
-            const float inv = __frcp_rn(qW);
+            const float inv = __frcp_rn(total[wib][lane][C]) * Fmt<DT>::UNIT;
             float res[C];
 #pragma unroll
-            for (int c = 0; c < C; ++c) res[c] = qacc[c] * inv;
+            for (int c = 0; c < C; ++c) res[c] = total[wib][lane][c] * inv;
             store_out<C>(p.out, i, res);
         }
         __syncwarp();

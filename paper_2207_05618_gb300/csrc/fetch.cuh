@@ -10,6 +10,7 @@
 #include <cuda_fp8.h>
 
 #include "htex_internal.h"
+#include "packed.cuh"
 
 namespace htex {
 
@@ -119,6 +120,17 @@ __device__ __forceinline__ float dec1(uint32_t b) {
 // an integer-to-float conversion on the slower conversion pipe.
 __device__ __forceinline__ float byte_as_float(uint32_t word, int c) {
     return __uint_as_float(__byte_perm(word, 0x4B000000u, 0x7540u | uint32_t(c))) - 8388608.0f;
+}
+
+// Four bytes of a packed word as floats, the same way, two channels per add.
+__device__ __forceinline__ void bytes_as_floats(uint32_t word, float (&t)[4]) {
+    const uint64_t bias = pack2(-8388608.0f, -8388608.0f);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const uint64_t v = add2(pack2(__uint_as_float(__byte_perm(word, 0x4B000000u, 0x7540u + 2 * k)),
+                                      __uint_as_float(__byte_perm(word, 0x4B000000u, 0x7541u + 2 * k))), bias);
+        unpack2(v, t[2 * k], t[2 * k + 1]);
+    }
 }
 
 // Channel c of a packed 8-bit-per-channel texel word, decoded.
@@ -263,6 +275,8 @@ struct Raw {
                     t[2] = hi.x;
                     t[3] = hi.y;
                 }
+            } else if constexpr (DT == HTEX_U8 && C == 4) {
+                bytes_as_floats(a, t);
             } else {
 #pragma unroll
                 for (int c = 0; c < C; ++c) t[c] = dec_byte<DT>(a, c);

@@ -153,3 +153,37 @@ def test_sorted_aniso_equals_unsorted_multi_chunk():
     sel = np.random.default_rng(17).choice(n, 20000, replace=False)
     _cmp(b.cpu().numpy().astype(np.float64)[sel],
          oracle.lookup_aniso(mo, to, tuple(x[sel] for x in qs), 16, nthreads=8), _tol(16, nmax=32))
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 129, 5000])
+def test_aniso_probe_intervals_and_warp_mates(n):
+    """Queries whose probe line is where the interval arithmetic can go
+    wrong: axes along u, along v, along the third side, zero and tiny axes,
+    centres on the triangle's sides and corners, 16 probes that stay inside,
+    leave or never reach a neighbouring quad, beside invalid queries; ragged
+    counts around a warp and a block.  Against the oracle, and bit for bit
+    against the same queries in another order (other warp mates)."""
+    gen = lambda: syn.cylinder(around=12, rows=5, seed=21)
+    mo, to, tl = _case(gen, lambda E: (np.arange(E) * 5 % 7).astype(np.int32), 4, "u8",
+                       hx.BUILD_MIPS | hx.MIRROR_BOUNDARY, seed=22)
+    rng = np.random.default_rng(n)
+    h, u, v = rng.integers(0, mo.H, n).astype(np.int32), rng.random(n), rng.random(n)
+    side = rng.integers(0, 8, n)
+    u = np.where(side == 0, 0.0, np.where(side == 1, 1.0, u))
+    v = np.where((side == 1) | (side == 2), 0.0, np.where(side == 3, 1.0 - u, v))
+    u, v = np.where(u + v > 1, 1 - u, u), np.where(u + v > 1, 1 - v, v)
+    major = np.exp2(rng.uniform(-14, 3, n))
+    minor = major / np.array([1.0, 3.0, 15.9, 16.0, 40.0])[rng.integers(0, 5, n)]
+    th = np.array([0.0, 0.5, 1.0, -0.25, 0.25, 0.1])[rng.integers(0, 6, n)] * np.pi
+    c, s = np.cos(th), np.sin(th)
+    c, s = np.where(np.abs(c) < 1e-9, 0.0, c), np.where(np.abs(s) < 1e-9, 0.0, s)
+    d = [major * c, major * s, -minor * s, minor * c]
+    flat = rng.integers(0, 6, n)
+    d = [np.where(flat == 0, 0.0, x).astype(np.float32) for x in d]        # both axes zero
+    d[2], d[3] = np.where(flat == 1, 0.0, d[2]), np.where(flat == 1, 1e-30, d[3])   # a degenerate minor axis
+    h = np.where(rng.random(n) < 0.05, -1, h).astype(np.int32)
+    qs = tuple(np.asarray(x, np.int32 if k == 0 else np.float32) for k, x in enumerate([h, u, v] + d))
+    got = _gpu(tl, qs, 16)
+    _cmp(got, oracle.lookup_aniso(mo, to, qs, 16), _tol(16, nmax=64))
+    perm = rng.permutation(n)
+    np.testing.assert_array_equal(_gpu(tl, tuple(x[perm] for x in qs), 16), got[perm])
