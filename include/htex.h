@@ -424,8 +424,8 @@ htex_status htex_triangle_vertices(const htex_geometry* g, float* out, htex_stre
  *              per pixel; h = -1 (an invalid query) where nothing is seen
  *   depth      device [height][width] float, nullable: NDC depth (NaN if empty)
  * Triangles with a vertex at or behind the camera plane (w <= 0) are not
- * drawn.  Scratch (8 bytes per pixel) comes stream-ordered from a
- * library-owned pool.  Asynchronous. */
+ * drawn.  Scratch (8 bytes per pixel and 64 per halfedge) comes
+ * stream-ordered from a library-owned pool.  Asynchronous. */
 htex_status htex_rasterize(const htex_geometry* g, const float* view_proj, int32_t width, int32_t height,
                            htex_query* queries, float* depth, htex_stream stream);
 

@@ -157,3 +157,29 @@ def test_displacement_formats_and_block_edges(dtype, C, channel, T):
     got = render.Geometry(mesh, pos).displace(tl, T, 0.3, channel=channel).cpu().numpy()
     pos32 = pos.astype(np.float32).astype(np.float64)
     np.testing.assert_allclose(got, oracle.displace(mo, to, pos32, T, 0.3, channel=channel), atol=2e-5)
+
+
+@pytest.mark.parametrize("W,H,eye", [(33, 31, 2.6), (257, 190, 1.9), (640, 3, 2.2), (1, 200, 2.2)])
+def test_rasterizer_small_and_large_boxes(W, H, eye):
+    """Bounding boxes on both sides of the 1024 pixels that a warp pools
+    (a cube's 24 large triangles beside a fine sphere's, one mesh), boxes
+    one pixel wide or high, boxes cut by the frame, and a last warp that is
+    not full: clear pixels carry the oracle's halfedge and depth."""
+    fs, fv, V, pos = syn.cube()
+    fs2, fv2, V2, pos2 = syn.uv_sphere(slices=40, rings=30, seed=3)
+    fs, fv = np.concatenate([fs, fs2]), np.concatenate([fv, fv2 + V])
+    pos = np.concatenate([pos - 0.5, pos2 * 0.3 + [0.9, 0.2, 0.1]])
+    mo = oracle.mesh_from_faces(fs, fv, V + V2)
+    M = syn.perspective(50.0, W / H, 0.3, 10.0) @ syn.look_at([eye, -0.4, 0.5], [0, 0, 0], [0, 0, 1])
+    g = render.Geometry(hx.Mesh(fs, fv, V + V2), pos)
+    assert g.H % 32 != 0 or g.H > 256
+    depth = torch.empty(W * H, dtype=torch.float32, device="cuda")
+    gh = g.rasterize(M, W, H, depth=depth).cpu().numpy()[:, 0].reshape(H, W)
+    pos32 = pos.astype(np.float32).astype(np.float64)
+    hh, _, _, _, dref, margin, gap = oracle.rasterize(mo, pos32, M.astype(np.float32).astype(np.float64), W, H)
+    clear = (hh >= 0) & (margin > 1e-3) & (gap > 1e-4)
+    assert clear.sum() > 0
+    np.testing.assert_array_equal(gh[clear], hh[clear])
+    np.testing.assert_allclose(depth.cpu().numpy().reshape(H, W)[clear], dref[clear], atol=1e-5)
+    empty = gh < 0
+    assert np.all((hh[empty] < 0) | (margin[empty] < 1e-3))
