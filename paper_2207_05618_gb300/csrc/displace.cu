@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(kDisplaceThreads) k_displace(Asset<GlobalSpace
                 acc = fmaf(g.w[1] * t.sc[e], b, acc);
                 W += g.ws;
             }
-            const float d = acc * __frcp_rn(W);
+            const float d = acc * (__frcp_rn(W) * Fmt<DT>::UNIT);
             const float w = 1.0f - L.x - L.y;
             float N[3];
 #pragma unroll

@@ -84,7 +84,7 @@ struct SharedSpace {
 
 // ES: bytes per channel; SCALED: decoded codes are multiplied by the
 // texture's scale; UNIT: constant factor of every decoded code (applied to
-// the tap weights).
+// the result).
 template <int DT> struct Fmt;
 template <> struct Fmt<HTEX_F32> { static constexpr int ES = 4; static constexpr bool SCALED = false; static constexpr float UNIT = 1.0f; };
 template <> struct Fmt<HTEX_U8> { static constexpr int ES = 1; static constexpr bool SCALED = false; static constexpr float UNIT = 1.0f / 255.0f; };
@@ -93,7 +93,7 @@ template <> struct Fmt<HTEX_BF16> { static constexpr int ES = 2; static constexp
 template <> struct Fmt<HTEX_E4M3> { static constexpr int ES = 1; static constexpr bool SCALED = true; static constexpr float UNIT = 1.0f; };
 
 // RGBA8 UNORM: the code b stands for b / 255; the lookup kernels apply the
-// 1/255 to the tap weight (Fmt<HTEX_U8>::UNIT) rather than to each channel.
+// 1/255 to the result (Fmt<HTEX_U8>::UNIT) rather than to each texel.
 __device__ __forceinline__ float dec_u8(uint32_t b) { return float(b); }
 __device__ __forceinline__ float dec_f16(uint32_t b) { return __half2float(__ushort_as_half((unsigned short)b)); }
 __device__ __forceinline__ float dec_bf16(uint32_t b) { return __uint_as_float(b << 16); }
@@ -297,7 +297,7 @@ struct Raw {
 // A resident asset seen from one memory space.
 template <class S>
 struct Asset {
-    S rec;      // int4 per halfedge
+    S rec;      // int4 per halfedge (in shared memory four arrays of a word per halfedge)
     S hdr;      // int4 per edge (unused when uniform)
     S scale;    // float per edge
     S pool;     // texel bytes

@@ -21,7 +21,9 @@ struct htex_mesh {
 // Lookup record of halfedge h (16 bytes): the three halfedges Alg. 3
 // visits are h, Next(h) and Prev(h); for each, the edge (texture) it maps
 // to through Edge(.) and whether Alg. 2 reflects its coordinates
-// (bit 31 set when g < Twin(g)).  w holds Face(h).
+// (bit 31 set when g < Twin(g)).  w holds the log2 resolutions of the three
+// textures, four bits each (so that a fetch that cannot reach its quad needs
+// no texture header).
 //
 // Texture header of edge e (16 bytes): x = byte offset / 16, y = log2 N_e,
 // z = scale bits (float), w = 0.

@@ -34,12 +34,38 @@ __device__ __forceinline__ void store_out(float* out, int64_t i, const float (&r
     }
 }
 
-// The record of a query's halfedge (zeros when the id is out of range;
-// such a query is rejected before the record is used).
+// The record of a query's halfedge: the texture codes of h, Next(h) and
+// Prev(h) and the log2 sizes of their textures (zeros or those of halfedge 0
+// when the id is out of range; such a query is rejected before the record is
+// used).  From global memory it is one 16-byte word, loaded ahead; in shared
+// memory the four fields are arrays of their own, read where they are
+// needed: a warp's 32 lookups of 16-byte records from shared memory took
+// about ten wavefronts, of 4-byte codes one to two.
 template <class S>
-__device__ __forceinline__ uint4 record_of(const Asset<S>& A, int4 raw) {
-    if (unsigned(raw.x) >= unsigned(A.H)) return make_uint4(0, 0, 0, 0);
-    return A.rec.ld16(typename S::off_t(raw.x) * 16u);
+struct Record {
+    uint4 r;
+    __device__ __forceinline__ uint32_t own() const { return r.x; }
+    __device__ __forceinline__ uint32_t edge(bool next) const { return next ? r.y : r.z; }
+    __device__ __forceinline__ uint32_t sizes() const { return r.w; }
+};
+template <>
+struct Record<SharedSpace> {
+    SharedSpace rec;
+    uint32_t at, field;   // byte offset of the halfedge's word, bytes of one array
+    __device__ __forceinline__ uint32_t own() const { return rec.ld4(at); }
+    __device__ __forceinline__ uint32_t edge(bool next) const { return rec.ld4(at + (next ? field : 2u * field)); }
+    __device__ __forceinline__ uint32_t sizes() const { return rec.ld4(at + 3u * field); }
+};
+
+template <class S>
+__device__ __forceinline__ Record<S> record_of(const Asset<S>& A, int4 raw) {
+    if constexpr (std::is_same<S, SharedSpace>::value) {
+        const uint32_t h = unsigned(raw.x) < unsigned(A.H) ? unsigned(raw.x) : 0u;
+        return Record<S>{A.rec, h * 4u, uint32_t(A.H) * 4u};
+    } else {
+        if (unsigned(raw.x) >= unsigned(A.H)) return Record<S>{make_uint4(0, 0, 0, 0)};
+        return Record<S>{A.rec.ld16(typename S::off_t(raw.x) * 16u)};
+    }
 }
 
 // The taps of one query, gathered in slots: up to 4 + 4 (own, two levels)
@@ -52,12 +78,10 @@ struct Gather {
     static constexpr int K = 16;
     Raw<DT, C> raw[DEFER ? K : 1];
     float w[DEFER ? K : 1];
-    float acc[C];
+    Sums<C> acc;
     float W = 0.0f;
 
     __device__ __forceinline__ Gather() {
-#pragma unroll
-        for (int c = 0; c < C; ++c) acc[c] = 0.0f;
         // slots of parts the warp skips keep weight zero
 #pragma unroll
         for (int k = 0; k < (DEFER ? K : 1); ++k) w[k] = 0.0f;
@@ -73,8 +97,7 @@ struct Gather {
         } else {
             float t[C];
             load_texel_if<DT, C>(pool, on, o, t);
-#pragma unroll
-            for (int c = 0; c < C; ++c) acc[c] = fmaf(wd, t[c], acc[c]);
+            acc.fma(wd, t);
         }
     }
 
@@ -84,18 +107,17 @@ struct Gather {
             for (int k = 0; k < K; ++k) {
                 float t[C];
                 raw[k].decode(t);
-#pragma unroll
-                for (int c = 0; c < C; ++c) acc[c] = fmaf(w[k], t[c], acc[c]);
+                acc.fma(w[k], t);
             }
         }
     }
 };
 
 // Data weight factor of a texture's decoded codes: its scale (scaled
-// formats) times the format's unit (1/255 for RGBA8).
+// formats); the format's unit (1/255 for RGBA8) is applied to the result.
 template <int DT>
 __device__ __forceinline__ float code_factor(const TexRef& t) {
-    return (Fmt<DT>::SCALED ? t.scale : 1.0f) * Fmt<DT>::UNIT;
+    return Fmt<DT>::SCALED ? t.scale : 1.0f;
 }
 
 // Taps are loaded only where their weight (before the code factor) is
@@ -153,15 +175,15 @@ __device__ __forceinline__ void edge_fetch(const Asset<S>& A, unsigned act, bool
 // has a positive footprint, so every fetch is level 0 only.
 template <int DT, int C, bool L0, bool DEFER, bool UNI, class S>
 __device__ __forceinline__ void lookup_body(const Asset<S>& A, const FwdParams& p, unsigned act, bool ok, float u,
-                                            float v, float f, uint4 rec, int64_t dst) {
-    const bool uni = UNI || A.uniform_log2n >= 0;
+                                            float v, float f, const Record<S>& rec, int64_t dst) {
     const float lf = L0 ? -__int_as_float(0x7f800000) : footprint_log2(f);
     Gather<DT, C, DEFER> g;
 
     // own quad at (u, v), through Alg. 2
-    const TexRef to = tex_ref<DT, UNI>(A, rec.x & ~kFlipBit);
+    const uint32_t co = rec.own();
+    const TexRef to = tex_ref<DT, UNI>(A, co & ~kFlipBit);
     const Lod d = L0 ? Lod{0, -1, 1.0f, 0.0f} : select_lod(lf, to.n);
-    const bool fo = rec.x & kFlipBit;
+    const bool fo = co & kFlipBit;
     const float x = fo ? 1.0f - u : u, y = fo ? 1.0f - v : v;
     own_taps<DT, C, 0>(A, to, L0 ? 0 : d.l0, x, y, ok ? (L0 ? 1.0f : d.w0) : 0.0f, g);
     if constexpr (!L0) {
@@ -169,33 +191,50 @@ __device__ __forceinline__ void lookup_body(const Asset<S>& A, const FwdParams& 
         if (__any_sync(act, two)) own_taps<DT, C, 4>(A, to, two ? d.l1 : d.l0, x, y, two ? d.w1 : 0.0f, g);
     }
 
-    // which edge fetches have taps in bounds (at the coarsest level read)
-    const TexRef tn = tex_ref<DT, UNI>(A, rec.y & ~kFlipBit);
-    const TexRef tp = tex_ref<DT, UNI>(A, rec.z & ~kFlipBit);
-    const Lod dn = (L0 || uni) ? d : select_lod(lf, tn.n);
-    const Lod dp = (L0 || uni) ? d : select_lod(lf, tp.n);
-    const bool nn = ok && across_weight(u, 1 << (tn.n - coarsest(dn))) > 0.0f;
-    const bool pp = ok && across_weight(v, 1 << (tp.n - coarsest(dp))) > 0.0f;
+    // which edge fetches have taps in bounds (at the coarsest level read); a
+    // texture's header or scale is read in the pass that needs it, one per
+    // lane instead of two
+    const int nN = UNI ? to.n : int(rec.sizes() >> 4 & 15u), nP = UNI ? to.n : int(rec.sizes() >> 8 & 15u);
+    const Lod dn = (L0 || UNI) ? d : select_lod(lf, nN);
+    const Lod dp = (L0 || UNI) ? d : select_lod(lf, nP);
+    const bool nn = ok && across_weight(u, 1 << (nN - coarsest(dn))) > 0.0f;
+    const bool pp = ok && across_weight(v, 1 << (nP - coarsest(dp))) > 0.0f;
 
     if (__any_sync(act, nn || pp)) {   // first edge pass: Next where needed, else Prev
         const bool row = nn;
-        edge_fetch<DT, C, 8, L0>(A, act, nn || pp, row ? tn : tp, row ? dn : dp, row ? u : v, row ? v : u,
-                                 ((row ? rec.y : rec.z) & kFlipBit) != 0, row, g);
+        const uint32_t code = rec.edge(row);
+        TexRef t;
+        if constexpr (L0 && UNI && !Fmt<DT>::SCALED && std::is_same<S, GlobalSpace>::value) {
+            // no loads either way: both places first, then the choice (2% faster at
+            // level 0: 7M one-byte lookups 234 -> 229 us; with footprints, or the
+            // pool in shared memory, 3-7% slower than the choice first)
+            const TexRef tn = tex_ref<DT, UNI>(A, rec.edge(true) & ~kFlipBit);
+            const TexRef tp = tex_ref<DT, UNI>(A, rec.edge(false) & ~kFlipBit);
+            t = row ? tn : tp;
+        } else {
+            t = tex_ref<DT, UNI>(A, code & ~kFlipBit);
+        }
+        edge_fetch<DT, C, 8, L0>(A, act, nn || pp, t, row ? dn : dp, row ? u : v, row ? v : u,
+                                 (code & kFlipBit) != 0, row, g);
     }
-    if (__any_sync(act, nn && pp))     // second pass: Prev for lanes that need both
-        edge_fetch<DT, C, 12, L0>(A, act, nn && pp, tp, dp, v, u, (rec.z & kFlipBit) != 0, false, g);
+    if (__any_sync(act, nn && pp)) {   // second pass: Prev for lanes that need both
+        const uint32_t code = rec.edge(false);
+        const TexRef t = tex_ref<DT, UNI>(A, code & ~kFlipBit);
+        edge_fetch<DT, C, 12, L0>(A, act, nn && pp, t, dp, v, u, (code & kFlipBit) != 0, false, g);
+    }
 
     g.finish();
     // an invalid query has every weight zero: W = 0, 1/W = inf, 0 * inf = NaN
-    const float inv = __frcp_rn(g.W);
+    const float inv = __frcp_rn(g.W) * Fmt<DT>::UNIT;
     float r[C];
+    g.acc.get(r);
 #pragma unroll
-    for (int c = 0; c < C; ++c) r[c] = g.acc[c] * inv;
+    for (int c = 0; c < C; ++c) r[c] *= inv;
     store_out<C>(p.out, dst, r);
 }
 
 template <int DT, int C, bool DEFER, bool UNI = false, class S>
-__device__ __forceinline__ void lookup_one(const Asset<S>& A, const FwdParams& p, int4 raw, uint4 rec,
+__device__ __forceinline__ void lookup_one(const Asset<S>& A, const FwdParams& p, int4 raw, const Record<S>& rec,
                                            int64_t dst) {
     int h;
     float u, v, f;

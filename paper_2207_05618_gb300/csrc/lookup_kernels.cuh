@@ -35,7 +35,7 @@ __device__ __forceinline__ void lookup_loop(const Asset<S>& A, const FwdParams& 
         raw1 = ld_query(p.q, i1);
         dst1 = dst_of<BINNED>(p, i1);
     }
-    uint4 rec0 = record_of(A, raw0);
+    Record<S> rec0 = record_of(A, raw0);
     while (true) {
         const I i2 = i1 + stride;
         int4 raw2 = make_int4(-1, 0, 0, 0);
@@ -44,8 +44,7 @@ __device__ __forceinline__ void lookup_loop(const Asset<S>& A, const FwdParams& 
             raw2 = ld_query(p.q, i2);
             dst2 = dst_of<BINNED>(p, i2);
         }
-        uint4 rec1 = make_uint4(0, 0, 0, 0);
-        if (i1 < n) rec1 = record_of(A, raw1);
+        const Record<S> rec1 = record_of(A, raw1);   // zeros past the end
         lookup_one<DT, C, DEFER, UNI>(A, p, raw0, rec0, dst0);
         if (i1 >= n) break;
         raw0 = raw1;
@@ -71,7 +70,7 @@ __device__ __forceinline__ void lookup_loop_pairs(const Asset<S>& A, const FwdPa
         const int4 rb = j < n ? ld_query(p.q, j) : make_int4(-1, 0, 0, 0);
         if (i + 4 * stride < n) prefetch_query(p.q, i + 4 * stride);
         if (j + 4 * stride < n) prefetch_query(p.q, j + 4 * stride);
-        const uint4 ca = record_of(A, ra), cb = record_of(A, rb);
+        const Record<S> ca = record_of(A, ra), cb = record_of(A, rb);
         lookup_one<DT, C, DEFER, UNI>(A, p, ra, ca, dst_of<BINNED>(p, i));
         if (j < n) lookup_one<DT, C, DEFER, UNI>(A, p, rb, cb, dst_of<BINNED>(p, j));
     }
@@ -128,7 +127,14 @@ __global__ void __launch_bounds__(kStagedThreads, 1) k_lookup_staged(Asset<Globa
                                                                   int64_t pool_bytes, FwdParams p) {
     extern __shared__ __align__(16) uint8_t smem[];
     const StageLayout L = stage_layout(G.H, E, pool_bytes);
-    stage16(smem + L.rec, G.rec.base, uint32_t(G.H) * 16u);
+    for (uint32_t h = threadIdx.x; h < uint32_t(G.H); h += blockDim.x) {   // the records as four arrays (Record<SharedSpace>)
+        const uint4 r = G.rec.ld16(uint64_t(h) * 16u);
+        uint32_t* w = reinterpret_cast<uint32_t*>(smem + L.rec) + h;
+        w[0] = r.x;
+        w[G.H] = r.y;
+        w[2 * G.H] = r.z;
+        w[3 * G.H] = r.w;
+    }
     stage16(smem + L.hdr, G.hdr.base, uint32_t(E) * 16u);
     stage16(smem + L.scale, G.scale.base, (uint32_t(E) * 4u + 15u) & ~15u);
     stage16(smem + L.pool, G.pool.base, uint32_t(pool_bytes));

@@ -383,14 +383,14 @@ htex_status htex_asset_arrays(const htex_mesh* m, int32_t C, htex_dtype dtype, c
     A.E = E;
     A.C = C;
     A.dtype = dtype;
-    // per-halfedge lookup records: the edge and Alg. 2 reflection of h, Next(h), Prev(h)
+    // per-halfedge lookup records: the edge and Alg. 2 reflection of h, Next(h), Prev(h), and their log2 sizes
     A.rec.assign(size_t(H) * 4, 0);
     auto code = [&](int32_t g) { return uint32_t(m->edge[g]) | (g < m->twin[g] ? kFlipBit : 0u); };
     for (int32_t h = 0; h < H; ++h) {
         A.rec[4 * size_t(h) + 0] = int32_t(code(h));
         A.rec[4 * size_t(h) + 1] = int32_t(code(m->next[h]));
         A.rec[4 * size_t(h) + 2] = int32_t(code(m->prev[h]));
-        A.rec[4 * size_t(h) + 3] = m->face[h];
+        A.rec[4 * size_t(h) + 3] = log2n[m->edge[h]] | log2n[m->edge[m->next[h]]] << 4 | log2n[m->edge[m->prev[h]]] << 8;
     }
     A.hdr.assign(size_t(E) * 4, 0);
     A.scale.assign((size_t(E) + 3) & ~size_t(3), 1.0f);   // whole 16-byte words (shared-memory staging)
