@@ -34,10 +34,16 @@ def _ptr(a: np.ndarray):
 def _stream(stream):
     if stream is None:
         import torch
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+        # the raw handle without a Stream object around it (torch's own
+        # generated code takes it the same way): a third of the host time of
+        # a small lookup's call
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is not None and torch.cuda.is_initialized():
+            return raw(torch.cuda.current_device())
+        return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
-        return ctypes.c_void_p(stream)
-    return ctypes.c_void_p(stream.cuda_stream)
+        return stream
+    return stream.cuda_stream
 
 
 class Mesh:
@@ -174,7 +180,7 @@ class Textures:
             if not src.is_contiguous():
                 raise ValueError("src must be contiguous")
             nbytes = src.numel() * src.element_size()
-            ptr = ctypes.c_void_p(src.data_ptr())
+            ptr = src.data_ptr()
         else:
             arr = np.ascontiguousarray(src)
             nbytes, ptr = arr.nbytes, _ptr(arr)
@@ -194,7 +200,7 @@ class Textures:
             if not (isinstance(x, torch.Tensor) and x.is_cuda and x.dtype == torch.float32 and x.is_contiguous()
                     and x.numel() == self.pool_elements):
                 raise ValueError(f"{name} must be a contiguous float32 CUDA tensor of pool_elements")
-        ptrs = [ctypes.c_void_p(x.data_ptr() if x is not None else None) for x in (master, grad, m, v)]
+        ptrs = [x.data_ptr() if x is not None else None for x in (master, grad, m, v)]
         check(self._lib.htex_textures_adam_step(self._h, *ptrs,
                                                 self.pool_elements, float(lr), float(betas[0]), float(betas[1]),
                                                 float(eps), int(step), _stream(stream)), "htex_textures_adam_step")
@@ -229,7 +235,7 @@ def _check_tensor(t, name, dtype, cols):
     import torch
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
-    if t.dtype != dtype or not t.is_contiguous() or t.dim() != 2 or t.shape[1] != cols:
+    if t.dtype != dtype or t.dim() != 2 or t.size(1) != cols or not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous {dtype} [n, {cols}]")
 
 
@@ -242,8 +248,8 @@ def lookup(tex: Textures, queries, out=None, flags: int = 0, stream=None, status
         out = torch.empty((n, tex.channels), dtype=torch.float32, device=queries.device)
     else:
         _check_tensor(out, "out", torch.float32, tex.channels)
-    st = ctypes.c_void_p(status.data_ptr()) if status is not None else None
-    check(tex._lib.htex_lookup(tex._h, ctypes.c_void_p(queries.data_ptr()), n, ctypes.c_void_p(out.data_ptr()),
+    st = status.data_ptr() if status is not None else None
+    check(tex._lib.htex_lookup(tex._h, queries.data_ptr(), n, out.data_ptr(),
                                int(flags), _stream(stream), st), "htex_lookup")
     return out
 
@@ -267,9 +273,9 @@ def lookup_aniso(tex: Textures, queries, max_aniso: int = 16, out=None, stream=N
         out = torch.empty((n, tex.channels), dtype=torch.float32, device=queries.device)
     else:
         _check_tensor(out, "out", torch.float32, tex.channels)
-    st = ctypes.c_void_p(status.data_ptr()) if status is not None else None
-    check(tex._lib.htex_lookup_aniso(tex._h, ctypes.c_void_p(queries.data_ptr()), n, int(max_aniso), int(flags),
-                                     ctypes.c_void_p(out.data_ptr()), _stream(stream), st), "htex_lookup_aniso")
+    st = status.data_ptr() if status is not None else None
+    check(tex._lib.htex_lookup_aniso(tex._h, queries.data_ptr(), n, int(max_aniso), int(flags),
+                                     out.data_ptr(), _stream(stream), st), "htex_lookup_aniso")
     return out
 
 
@@ -287,8 +293,8 @@ def sort_queries(tex: Textures, queries, sorted_queries=None, pos=None, stream=N
         pos = torch.empty(n, dtype=torch.int32, device=queries.device)
     if not (pos.is_cuda and pos.dtype == torch.int32 and pos.is_contiguous() and pos.numel() == n):
         raise ValueError("pos must be a contiguous CUDA int32 tensor of n elements")
-    check(tex._lib.htex_queries_sort(tex._h, ctypes.c_void_p(queries.data_ptr()), n,
-                                     ctypes.c_void_p(sorted_queries.data_ptr()), ctypes.c_void_p(pos.data_ptr()),
+    check(tex._lib.htex_queries_sort(tex._h, queries.data_ptr(), n,
+                                     sorted_queries.data_ptr(), pos.data_ptr(),
                                      _stream(stream)), "htex_queries_sort")
     return sorted_queries, pos
 
@@ -307,8 +313,8 @@ def gather_results(sorted_out, pos, out=None, stream=None):
     else:
         _check_tensor(out, "out", torch.float32, c)
     lib = load()
-    check(lib.htex_results_gather(ctypes.c_void_p(sorted_out.data_ptr()), ctypes.c_void_p(pos.data_ptr()), n, c,
-                                  ctypes.c_void_p(out.data_ptr()), _stream(stream)), "htex_results_gather")
+    check(lib.htex_results_gather(sorted_out.data_ptr(), pos.data_ptr(), n, c,
+                                  out.data_ptr(), _stream(stream)), "htex_results_gather")
     return out
 
 
@@ -325,8 +331,8 @@ def lookup_host(tex: Textures, queries, out=None, flags: int = 0, stream=None, s
         out = torch.empty((n, tex.channels), dtype=torch.float32, pin_memory=True)
     if out.is_cuda or out.dtype != torch.float32 or tuple(out.shape) != (n, tex.channels) or not out.is_contiguous():
         raise ValueError("out must be a contiguous host float32 [n, channels] tensor")
-    st = ctypes.c_void_p(status.data_ptr()) if status is not None else None
-    check(tex._lib.htex_lookup_host(tex._h, ctypes.c_void_p(qt.data_ptr()), n, ctypes.c_void_p(out.data_ptr()),
+    st = status.data_ptr() if status is not None else None
+    check(tex._lib.htex_lookup_host(tex._h, qt.data_ptr(), n, out.data_ptr(),
                                     int(flags), _stream(stream), st), "htex_lookup_host")
     return out
 
@@ -339,10 +345,10 @@ def lookup_backward(tex: Textures, queries, grad_out, grad_texels=None, flags: i
     _check_tensor(grad_out, "grad_out", torch.float32, tex.channels)
     if grad_texels is None:
         grad_texels = torch.zeros(tex.pool_elements, dtype=torch.float32, device=queries.device)
-    st = ctypes.c_void_p(status.data_ptr()) if status is not None else None
-    check(tex._lib.htex_lookup_backward(tex._h, ctypes.c_void_p(queries.data_ptr()), queries.shape[0],
-                                        ctypes.c_void_p(grad_out.data_ptr()),
-                                        ctypes.c_void_p(grad_texels.data_ptr()), int(flags), _stream(stream),
+    st = status.data_ptr() if status is not None else None
+    check(tex._lib.htex_lookup_backward(tex._h, queries.data_ptr(), queries.shape[0],
+                                        grad_out.data_ptr(),
+                                        grad_texels.data_ptr(), int(flags), _stream(stream),
                                         st), "htex_lookup_backward")
     return grad_texels
 

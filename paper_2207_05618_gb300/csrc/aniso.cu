@@ -379,10 +379,8 @@ __global__ void __launch_bounds__(kAnisoThreads, kAnisoBlocks) k_lookup_aniso(As
 
 template <int DT, int C>
 htex_status launch_aniso_c(const htex_textures* t, const AnisoParams& p, cudaStream_t s) {
-    int b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_lookup_aniso<DT, C>, kAnisoThreads, 0) != cudaSuccess ||
-        b < 1)
-        b = 1;
+    static Occupancy occupancy;
+    const int b = occupancy.get(k_lookup_aniso<DT, C>, kAnisoThreads, t->device);
     const int64_t want = (p.n + kAnisoThreads - 1) / kAnisoThreads;
     const int64_t grid = std::min<int64_t>(want, int64_t(t->num_sms) * b);
     k_lookup_aniso<DT, C><<<unsigned(grid), kAnisoThreads, 0, s>>>(global_asset(t), p);

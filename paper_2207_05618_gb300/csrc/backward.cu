@@ -382,8 +382,8 @@ template <int DT, int C, bool AGG>
 htex_status launch_bwd(const htex_textures* t, const BwdParams& p, cudaStream_t s) {
     const Asset<GlobalSpace> A = global_asset(t);
     auto k = k_backward<DT, C, AGG>;
-    int b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k, kThreads, 0) != cudaSuccess || b < 1) b = 1;
+    static Occupancy occupancy;
+    const int b = occupancy.get(k, kThreads, t->device);
     const int64_t want = (p.n + kThreads - 1) / kThreads;
     const int64_t grid = std::min<int64_t>(want, int64_t(t->num_sms) * b);
     k<<<unsigned(grid), kThreads, 0, s>>>(A, p);

@@ -177,9 +177,8 @@ __global__ void __launch_bounds__(kDisplaceThreads) k_displace(Asset<GlobalSpace
 
 template <int DT>
 htex_status launch_displace(const Asset<GlobalSpace>& A, const DisplaceParams& p, cudaStream_t s) {
+    // at most 37 KiB with the stage (T = 64: 2145 points, one triangle; T = 1: 256 triangles)
     const size_t smem = size_t(p.K) * sizeof(float4) + size_t(p.per_block) * sizeof(DisplaceTriangle);
-    if (cudaFuncSetAttribute(k_displace<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
-        return HTEX_ERR_CUDA;
     const unsigned grid = unsigned((A.H + p.per_block - 1) / p.per_block);
     k_displace<DT><<<grid, kDisplaceThreads, smem, s>>>(A, p);
     return cudaGetLastError() == cudaSuccess ? HTEX_OK : HTEX_ERR_CUDA;

@@ -1,6 +1,8 @@
 // Internal declarations of libhtex (not part of the public ABI).
 #pragma once
 
+#include <atomic>
+#include <cstddef>
 #include <cstdint>
 #include <vector>
 
@@ -105,6 +107,30 @@ cudaMemPool_t htex_scratch_pool(int device);
 // log2 of the halfedges per sort range so that a range's textures take
 // about 32 MB; -1 when the pool is too small for sorting to pay (lookup.cu).
 int htex_bin_shift(const htex_textures* t);
+
+// Resident blocks per SM of one kernel at one block size, asked of the
+// driver once per device (a property of the compiled kernel and the device;
+// the query takes longer than preparing the launch).  A kernel that needs
+// more than the default dynamic shared memory has its limit raised on the
+// same occasion.  One static object per kernel; threads may race to fill it,
+// with the same value.
+struct Occupancy {
+    static constexpr int kDevices = 64;
+    std::atomic<int> blocks[kDevices];
+
+    // 0: the shared-memory limit could not be raised
+    template <class K>
+    int get(K kernel, int threads, int device, size_t smem = 0) {
+        const bool known = device >= 0 && device < kDevices;
+        int b = known ? blocks[device].load(std::memory_order_relaxed) : 0;
+        if (b > 0) return b;
+        if (smem > 0 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
+            return 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, threads, smem) != cudaSuccess || b < 1) b = 1;
+        if (known) blocks[device].store(b, std::memory_order_relaxed);
+        return b;
+    }
+};
 
 // Kernel launchers (lookup.cu, backward.cu).  They validate nothing: the
 // C-ABI entry points have checked every argument.

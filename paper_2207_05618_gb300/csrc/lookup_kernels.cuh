@@ -183,7 +183,9 @@ htex_status launch_fwd(const htex_textures* t, const FwdParams& p, uint32_t flag
     } else {
         auto k = t->uniform_log2n >= 0 ? k_lookup_global<DT, C, BINNED, true> : k_lookup_global<DT, C, BINNED, false>;
         const int64_t want = (p.n + kGlobalThreads - 1) / kGlobalThreads;
-        const int64_t grid = std::min<int64_t>(want, int64_t(t->num_sms) * resident_blocks(k, kGlobalThreads, 0));
+        static Occupancy occupancy[2];
+        const int blocks = occupancy[t->uniform_log2n >= 0].get(k, kGlobalThreads, t->device);
+        const int64_t grid = std::min<int64_t>(want, int64_t(t->num_sms) * blocks);
         k<<<unsigned(grid), kGlobalThreads, 0, s>>>(A, p);
     }
     return cudaGetLastError() == cudaSuccess ? HTEX_OK : HTEX_ERR_CUDA;

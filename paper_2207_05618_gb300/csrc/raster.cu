@@ -321,9 +321,15 @@ __global__ void k_resolve(Camera cam, const unsigned long long* vis, const float
 }
 
 int grid_for(int64_t n) {
-    int dev = 0, sms = 148;
+    static std::atomic<int> known[Occupancy::kDevices];
+    int dev = 0;
     cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const bool in = dev >= 0 && dev < Occupancy::kDevices;
+    int sms = in ? known[dev].load(std::memory_order_relaxed) : 0;
+    if (sms == 0) {
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 148;
+        else if (in) known[dev].store(sms, std::memory_order_relaxed);
+    }
     return int(std::min<int64_t>((n + kThreads - 1) / kThreads, int64_t(sms) * 8));
 }
 

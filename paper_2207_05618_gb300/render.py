@@ -24,7 +24,7 @@ class Geometry:
     def triangle_vertices(self, stream=None):
         import torch
         out = torch.empty((self.H, 3, 3), dtype=torch.float32, device="cuda")
-        check(self._lib.htex_triangle_vertices(self._h, ctypes.c_void_p(out.data_ptr()), _stream(stream)),
+        check(self._lib.htex_triangle_vertices(self._h, out.data_ptr(), _stream(stream)),
               "htex_triangle_vertices")
         return out
 
@@ -34,9 +34,9 @@ class Geometry:
         m = np.ascontiguousarray(view_proj, np.float32).reshape(16)
         if queries is None:
             queries = torch.empty((width * height, 4), dtype=torch.int32, device="cuda")
-        dptr = ctypes.c_void_p(depth.data_ptr()) if depth is not None else None
+        dptr = depth.data_ptr() if depth is not None else None
         check(self._lib.htex_rasterize(self._h, m.ctypes.data_as(ctypes.c_void_p), int(width), int(height),
-                                       ctypes.c_void_p(queries.data_ptr()), dptr, _stream(stream)),
+                                       queries.data_ptr(), dptr, _stream(stream)),
               "htex_rasterize")
         return queries
 
@@ -47,9 +47,9 @@ class Geometry:
         m = np.ascontiguousarray(view_proj, np.float32).reshape(16)
         if queries is None:
             queries = torch.empty((width * height, 8), dtype=torch.int32, device="cuda")
-        dptr = ctypes.c_void_p(depth.data_ptr()) if depth is not None else None
+        dptr = depth.data_ptr() if depth is not None else None
         check(self._lib.htex_rasterize_aniso(self._h, m.ctypes.data_as(ctypes.c_void_p), int(width), int(height),
-                                             ctypes.c_void_p(queries.data_ptr()), dptr, _stream(stream)),
+                                             queries.data_ptr(), dptr, _stream(stream)),
               "htex_rasterize_aniso")
         return queries
 
@@ -58,7 +58,7 @@ class Geometry:
         K = (tess + 1) * (tess + 2) // 2
         out = torch.empty((self.H, K, 3), dtype=torch.float32, device="cuda")
         check(self._lib.htex_displace(self._h, tex._h, int(tess), float(scale), int(channel),
-                                      ctypes.c_void_p(out.data_ptr()), _stream(stream)), "htex_displace")
+                                      out.data_ptr(), _stream(stream)), "htex_displace")
         return out
 
     def close(self):
