@@ -241,8 +241,9 @@ void htex_textures_destroy(htex_textures* t);
 /* Filtered lookups (Section 4.4, Alg. 3 with Alg. 2), n queries.
  *   q         device [n] htex_query (16-byte aligned)
  *   out       device [n][channels] float (16-byte aligned when channels = 4)
- *   flags     HTEX_LOOKUP_BIN: when the pool exceeds 64 MiB, counting-sort
- *             the queries into ranges of consecutive halfedges first, in
+ *   flags     HTEX_LOOKUP_BIN: when the pool exceeds 64 MiB and n is at
+ *             least 2^18 (below, sorting costs more than it saves),
+ *             counting-sort the queries into ranges of consecutive halfedges first, in
  *             chunks of 2^24 queries, filter them in that order and gather
  *             the results back into query order (same results, bit for bit;
  *             scratch of 20 + 4 * channels bytes per chunk query,
@@ -277,11 +278,10 @@ htex_status htex_lookup(const htex_textures* t, const htex_query* q, int64_t n, 
  *   placed.
  *   q          device [n] htex_query_aniso (16-byte aligned)
  *   max_aniso  1..16
- *   flags      HTEX_LOOKUP_BIN: sort the queries by halfedge range first,
- *              as htex_lookup does (same results, bit for bit: each
- *              query's probes are summed in probe order whatever queries
- *              share its warp; scratch of 36 + 4 * channels bytes per
- *              chunk query)
+ *   flags      HTEX_LOOKUP_BIN: accepted; the queries are filtered in their
+ *              given order all the same (results never depend on the
+ *              order: each query's probes are summed in an order of its
+ *              own; sorting was slower at every size)
  *   out        device [n][channels] float (alignment as htex_lookup)
  *   d_status   device int32, nullable: incremented once per invalid query
  *              (h out of range, non-finite u, v or derivative, or an
@@ -352,7 +352,7 @@ htex_status htex_lookup_host(const htex_textures* t, const htex_query* q, int64_
  *   grad_texels  device float, one per pool element (pool_bytes / element
  *                size), same element order as the pool; accumulated into
  *                (the caller zeroes it); padding elements keep their values
- *   flags        HTEX_LOOKUP_BIN: when the pool exceeds 64 MiB, sort the
+ *   flags        HTEX_LOOKUP_BIN: when the pool exceeds 64 MiB (and n is at least 2^18), sort the
  *                queries as htex_lookup does (chunks of 2^24, ranges of
  *                consecutive halfedges; grad_out rows move with their
  *                queries) so that the threads resident together add into

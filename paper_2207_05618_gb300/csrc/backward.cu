@@ -384,9 +384,12 @@ htex_status launch_bwd(const htex_textures* t, const BwdParams& p, cudaStream_t 
     auto k = k_backward<DT, C, AGG>;
     static Occupancy occupancy;
     const int b = occupancy.get(k, kThreads, t->device);
-    const int64_t want = (p.n + kThreads - 1) / kThreads;
-    const int64_t grid = std::min<int64_t>(want, int64_t(t->num_sms) * b);
-    k<<<unsigned(grid), kThreads, 0, s>>>(A, p);
+    // a batch that does not fill every SM is spread over all of them, in
+    // blocks of fewer warps
+    const int64_t resident = int64_t(t->num_sms) * b;
+    const int threads = int(std::min<int64_t>(kThreads, ((p.n + resident - 1) / resident + 31) / 32 * 32));
+    const int64_t grid = std::min<int64_t>((p.n + threads - 1) / threads, resident);
+    k<<<unsigned(grid), threads, 0, s>>>(A, p);
     return cudaGetLastError() == cudaSuccess ? HTEX_OK : HTEX_ERR_CUDA;
 }
 

@@ -30,7 +30,6 @@
 #include <cuda_runtime.h>
 
 #include "lookup_kernels.cuh"
-#include "aniso_launch.h"
 
 namespace htex {
 
@@ -129,8 +128,8 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_scatter(const htex_query* q
 // ------------------------------------------ chunk-local sort (HTEX_LOOKUP_BIN)
 //
 // One chunk of m queries at a time: a bucket histogram, then per tile of
-// kSortThreads x kSortPer queries (fewer per thread for wider queries or a
-// payload) a local counting sort in shared memory, so that every
+// kSortThreads x kSortPer queries (half as many per thread with a payload)
+// a local counting sort in shared memory, so that every
 // bucket's run of the tile is written to the sorted copy as one contiguous
 // piece (whole sectors, not scattered 16-byte pieces), and each query's
 // sorted position is recorded in query order.  The lookup then filters the
@@ -141,12 +140,9 @@ constexpr int kSortThreads = 256;
 constexpr int kSortPer = 8;   // 16-byte query words per thread and tile (16: 8% slower sort, measured)
 constexpr int kSortMaxBuckets = 256;
 
-// QW: 16-byte words per query (1: htex_query, 2: htex_query_aniso); the
-// halfedge id is the first word's first int.
-template <int QW>
 __global__ void __launch_bounds__(kSortThreads) k_chunk_count(const int4* q, int64_t m, int32_t H, int shift,
                                                               uint32_t B, uint32_t* counts) {
-    constexpr int PER = kSortPer / QW, TILE = kSortThreads * PER;
+    constexpr int PER = kSortPer, TILE = kSortThreads * PER;
     __shared__ uint32_t hist[kSortMaxBuckets];
     for (uint32_t b = threadIdx.x; b < B; b += blockDim.x) hist[b] = 0;
     __syncthreads();
@@ -155,7 +151,7 @@ __global__ void __launch_bounds__(kSortThreads) k_chunk_count(const int4* q, int
 #pragma unroll
         for (int k = 0; k < PER; ++k) {
             const int64_t i = t0 + int64_t(k) * kSortThreads + threadIdx.x;
-            h[k] = i < m ? __ldg(reinterpret_cast<const int32_t*>(q + i * QW)) : 0;
+            h[k] = i < m ? __ldg(reinterpret_cast<const int32_t*>(q + i)) : 0;
         }
 #pragma unroll
         for (int k = 0; k < PER; ++k)
@@ -194,27 +190,27 @@ __device__ __forceinline__ void block_scan_buckets(const uint32_t* x, uint32_t* 
 
 // PC: floats of payload per query (rows of 'pay' in query order, moved to
 // 'spay' in sorted order with their queries); pos nullable.
-// Shared memory of k_chunk_scatter<QW, PC> (dynamic: a tile can exceed the
-// 48 KiB of static shared memory): the tile's queries (QW words each) and
-// payload rows, their buckets, and per bucket the first sorted position,
+// Shared memory of k_chunk_scatter<PC> (dynamic: a tile can exceed the
+// 48 KiB of static shared memory): the tile's queries and payload rows,
+// their buckets, and per bucket the first sorted position,
 // the tile's count, local offset and global base.
-template <int QW, int PC>
+template <int PC>
 struct ScatterSmem {
-    static constexpr int PER = kSortPer / QW / (PC > 0 ? 2 : 1), TILE = kSortThreads * PER;
+    static constexpr int PER = kSortPer / (PC > 0 ? 2 : 1), TILE = kSortThreads * PER;
     static constexpr size_t tile = 0;
-    static constexpr size_t pay = tile + size_t(TILE) * QW * 16;
+    static constexpr size_t pay = tile + size_t(TILE) * 16;
     static constexpr size_t bucket = pay + ((size_t(PC > 0 ? TILE * PC : 1) * 4 + 15) & ~size_t(15));
     static constexpr size_t arrays = bucket + ((size_t(TILE) * 2 + 15) & ~size_t(15));
     static constexpr size_t warps = arrays + size_t(4) * kSortMaxBuckets * 4;
     static constexpr size_t bytes = warps + (kSortThreads / 32) * 4;
 };
 
-template <int QW, int PC>
+template <int PC>
 __global__ void __launch_bounds__(kSortThreads) k_chunk_scatter(const int4* q, int64_t m, int32_t H, int shift,
                                                                 uint32_t B, const uint32_t* counts, uint32_t* taken,
                                                                 int4* sq, int32_t* pos, int32_t pos_base,
                                                                 const float* pay, float* spay) {
-    using L = ScatterSmem<QW, PC>;
+    using L = ScatterSmem<PC>;
     constexpr int PER = L::PER, TILE = L::TILE;
     extern __shared__ __align__(16) uint8_t smem[];
     int4* tile = reinterpret_cast<int4*>(smem + L::tile);
@@ -233,15 +229,13 @@ __global__ void __launch_bounds__(kSortThreads) k_chunk_scatter(const int4* q, i
         const int tm = int(min(int64_t(TILE), m - t0));
         for (uint32_t b = threadIdx.x; b < B; b += blockDim.x) cnt[b] = 0;
         __syncthreads();
-        int4 r[PER][QW];
+        int4 r[PER];
         float pv[PER][PC > 0 ? PC : 1];
         uint32_t bk[PER], rank[PER];
 #pragma unroll
         for (int k = 0; k < PER; ++k) {
             const int j = k * kSortThreads + threadIdx.x;
-#pragma unroll
-            for (int w = 0; w < QW; ++w)
-                if (j < tm) r[k][w] = __ldcs(q + (t0 + j) * QW + w);
+            if (j < tm) r[k] = __ldcs(q + t0 + j);
 #pragma unroll
             for (int c = 0; c < PC; ++c)
                 if (j < tm) pv[k][c] = __ldcs(pay + (t0 + j) * PC + c);
@@ -249,7 +243,7 @@ __global__ void __launch_bounds__(kSortThreads) k_chunk_scatter(const int4* q, i
 #pragma unroll
         for (int k = 0; k < PER; ++k) {
             if (k * kSortThreads + int(threadIdx.x) < tm) {
-                bk[k] = bucket_of(r[k][0].x, H, shift, B - 1);
+                bk[k] = bucket_of(r[k].x, H, shift, B - 1);
                 rank[k] = atomicAdd(&cnt[bk[k]], 1u);
             }
         }
@@ -263,8 +257,7 @@ __global__ void __launch_bounds__(kSortThreads) k_chunk_scatter(const int4* q, i
             const int j = k * kSortThreads + threadIdx.x;
             if (j < tm) {
                 const uint32_t lp = loff[bk[k]] + rank[k];
-#pragma unroll
-                for (int w = 0; w < QW; ++w) tile[lp * QW + w] = r[k][w];
+                tile[lp] = r[k];
 #pragma unroll
                 for (int c = 0; c < PC; ++c) tile_pay[lp * PC + c] = pv[k][c];
                 tile_bucket[lp] = uint16_t(bk[k]);
@@ -272,10 +265,9 @@ __global__ void __launch_bounds__(kSortThreads) k_chunk_scatter(const int4* q, i
             }
         }
         __syncthreads();
-        for (int x = threadIdx.x; x < tm * QW; x += kSortThreads) {   // one 16-byte word per thread
-            const int j = x / QW, w = x - j * QW;
+        for (int j = threadIdx.x; j < tm; j += kSortThreads) {
             const uint32_t b = tile_bucket[j];
-            sq[int64_t(gbase[b] + (uint32_t(j) - loff[b])) * QW + w] = tile[x];
+            sq[gbase[b] + (uint32_t(j) - loff[b])] = tile[j];
         }
         if constexpr (PC > 0) {
             for (int x = threadIdx.x; x < tm * PC; x += kSortThreads) {
@@ -357,6 +349,13 @@ constexpr int64_t kChunkBuckets = HTEX_CHUNK_BUCKETS;                // halfedge
 
 constexpr int64_t kBucketTexelBytes = int64_t(32) << 20;
 
+// Fewest queries HTEX_LOOKUP_BIN sorts.  Below, few queries share a texel
+// line whatever their order, and the sort's and gather's launches cost more
+// than they save: 16K / 128K / 256K random RGBA8 lookups on a 1.4 GB asset
+// take 26 / 30 / 34 us sorted, 8 / 20 / 29 us as they come (512K: 48 / 51,
+// 1M: 82 / 91); the adjoint 24 / 31 / 49 and 8 / 27 / 43 us.
+constexpr int64_t kMinSortedQueries = int64_t(1) << 18;
+
 template <bool BINNED>
 htex_status launch_fwd_dt(const htex_textures* t, const FwdParams& p, uint32_t flags, cudaStream_t s) {
     switch (t->dtype) {
@@ -426,23 +425,23 @@ size_t counter_bytes(const SortPlan& P) { return (size_t(2 * P.B) * 4 + 255) & ~
 // Sorts q[0..m) into sq within consecutive chunks of kSortChunk queries;
 // pos[i] = where query i went (nullable); PC floats of payload per query
 // follow their queries from pay to spay.  counters: counter_bytes(P) of
-// scratch.  QW: 16-byte words per query.
-template <int QW, int PC = 0>
+// scratch.
+template <int PC = 0>
 htex_status launch_sort(const htex_textures* t, const SortPlan& P, const int4* q, int64_t m, uint32_t* counters,
                         int4* sq, int32_t* pos, cudaStream_t s, const float* pay = nullptr, float* spay = nullptr) {
-    constexpr int64_t TILE = ScatterSmem<QW, PC>::TILE;
-    constexpr size_t smem = ScatterSmem<QW, PC>::bytes;
+    constexpr int64_t TILE = ScatterSmem<PC>::TILE;
+    constexpr size_t smem = ScatterSmem<PC>::bytes;
     static Occupancy occupancy;
-    const int resident = occupancy.get(k_chunk_scatter<QW, PC>, kSortThreads, t->device, smem);
+    const int resident = occupancy.get(k_chunk_scatter<PC>, kSortThreads, t->device, smem);
     if (resident == 0) return HTEX_ERR_CUDA;
     const int64_t blocks = int64_t(t->num_sms) * resident;
     for (int64_t c0 = 0; c0 < m; c0 += kSortChunk) {
         const int64_t mc = std::min<int64_t>(kSortChunk, m - c0);
         const int64_t g = std::min<int64_t>((mc + TILE - 1) / TILE, blocks);
         if (cudaMemsetAsync(counters, 0, size_t(2 * P.B) * 4, s) != cudaSuccess) return HTEX_ERR_CUDA;
-        k_chunk_count<QW><<<unsigned(g), kSortThreads, 0, s>>>(q + c0 * QW, mc, t->H, P.shift, P.B, counters);
-        k_chunk_scatter<QW, PC><<<unsigned(g), kSortThreads, smem, s>>>(
-            q + c0 * QW, mc, t->H, P.shift, P.B, counters, counters + P.B, sq + c0 * QW, pos ? pos + c0 : nullptr,
+        k_chunk_count<<<unsigned(g), kSortThreads, 0, s>>>(q + c0, mc, t->H, P.shift, P.B, counters);
+        k_chunk_scatter<PC><<<unsigned(g), kSortThreads, smem, s>>>(
+            q + c0, mc, t->H, P.shift, P.B, counters, counters + P.B, sq + c0, pos ? pos + c0 : nullptr,
             int32_t(c0), PC ? pay + c0 * PC : nullptr, PC ? spay + c0 * PC : nullptr);
         if (cudaGetLastError() != cudaSuccess) return HTEX_ERR_CUDA;
     }
@@ -473,7 +472,7 @@ htex_status launch_gather(const float* sout, const int32_t* pos, int64_t m, int 
 htex_status htex_launch_lookup(const htex_textures* t, const htex_query* q, int64_t n, float* out,
                                uint32_t flags, htex_stream stream, int32_t* d_status) {
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    if (!(flags & HTEX_LOOKUP_BIN) || htex_bin_shift(t) < 0)
+    if (!(flags & HTEX_LOOKUP_BIN) || htex_bin_shift(t) < 0 || n < kMinSortedQueries)
         return launch_fwd_dt<false>(t, FwdParams{q, n, out, d_status, nullptr}, flags, s);
 
     // one chunk at a time: sort, filter into the sorted copy, gather back
@@ -501,7 +500,7 @@ htex_status htex_launch_lookup(const htex_textures* t, const htex_query* q, int6
     htex_status st = HTEX_OK;
     for (int64_t c0 = 0; c0 < n && st == HTEX_OK; c0 += M) {
         const int64_t m = std::min<int64_t>(M, n - c0);
-        st = launch_sort<1>(t, P, words(q + c0), m, counters, words(sq), pos, s);
+        st = launch_sort<>(t, P, words(q + c0), m, counters, words(sq), pos, s);
         if (st == HTEX_OK) st = launch_fwd_dt<false>(t, FwdParams{sq, m, sout, d_status, nullptr}, fwd_flags, s);
         if (st == HTEX_OK) st = launch_gather(sout, pos, m, t->C, out + c0 * t->C, s);
     }
@@ -512,7 +511,7 @@ htex_status htex_launch_lookup(const htex_textures* t, const htex_query* q, int6
 template <int C>
 htex_status launch_sort_rows(const htex_textures* t, const SortPlan& P, const htex_query* q, int64_t m,
                              const float* g, uint32_t* counters, htex_query* sq, float* sg, cudaStream_t s) {
-    return launch_sort<1, C>(t, P, words(q), m, counters, words(sq), nullptr, s, g, sg);
+    return launch_sort<C>(t, P, words(q), m, counters, words(sq), nullptr, s, g, sg);
 }
 
 // The adjoint on sorted queries: each chunk sorted by halfedge range with
@@ -522,7 +521,8 @@ htex_status launch_sort_rows(const htex_textures* t, const SortPlan& P, const ht
 htex_status htex_launch_backward_sorted(const htex_textures* t, const htex_query* q, int64_t n,
                                         const float* grad_out, float* grad_texels, htex_stream stream,
                                         int32_t* d_status) {
-    if (htex_bin_shift(t) < 0) return htex_launch_backward(t, q, n, grad_out, grad_texels, 0u, stream, d_status);
+    if (htex_bin_shift(t) < 0 || n < kMinSortedQueries)
+        return htex_launch_backward(t, q, n, grad_out, grad_texels, 0u, stream, d_status);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const SortPlan P = sort_plan(t->H);
     const int64_t M = std::min<int64_t>(n, kSortChunk);
@@ -556,39 +556,6 @@ htex_status htex_launch_backward_sorted(const htex_textures* t, const htex_query
     return st;
 }
 
-htex_status htex_launch_aniso_sorted(const htex_textures* t, const htex_query_aniso* q, int64_t n, int32_t kmax,
-                                     float* out, htex_stream stream, int32_t* d_status) {
-    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    if (htex_bin_shift(t) < 0) return htex_launch_aniso(t, q, n, kmax, out, stream, d_status);
-    const SortPlan P = sort_plan(t->H);
-    const int64_t M = std::min<int64_t>(n, kSortChunk);
-    const size_t cnt_b = counter_bytes(P);
-    const size_t sq_b = size_t(M) * sizeof(htex_query_aniso), pos_b = (size_t(M) * 4 + 255) & ~size_t(255);
-    const size_t sout_b = size_t(M) * 4 * size_t(t->C);
-    cudaMemPool_t pool = htex_scratch_pool(t->device);
-    if (!pool) return HTEX_ERR_CUDA;
-    void* scratch = nullptr;
-    if (cudaMallocFromPoolAsync(&scratch, cnt_b + sq_b + pos_b + sout_b, pool, s) != cudaSuccess) {
-        cudaGetLastError();
-        return HTEX_ERR_OUT_OF_MEMORY;
-    }
-    uint8_t* base = static_cast<uint8_t*>(scratch);
-    uint32_t* counters = reinterpret_cast<uint32_t*>(base);
-    htex_query_aniso* sq = reinterpret_cast<htex_query_aniso*>(base + cnt_b);
-    int32_t* pos = reinterpret_cast<int32_t*>(base + cnt_b + sq_b);
-    float* sout = reinterpret_cast<float*>(base + cnt_b + sq_b + pos_b);
-    htex_status st = HTEX_OK;
-    for (int64_t c0 = 0; c0 < n && st == HTEX_OK; c0 += M) {
-        const int64_t m = std::min<int64_t>(M, n - c0);
-        st = launch_sort<2>(t, P, reinterpret_cast<const int4*>(q + c0), m, counters, reinterpret_cast<int4*>(sq),
-                            pos, s);
-        if (st == HTEX_OK) st = htex_launch_aniso(t, sq, m, kmax, sout, stream, d_status);
-        if (st == HTEX_OK) st = launch_gather(sout, pos, m, t->C, out + c0 * t->C, s);
-    }
-    cudaFreeAsync(scratch, s);
-    return st;
-}
-
 extern "C" htex_status htex_queries_sort(const htex_textures* t, const htex_query* q, int64_t n,
                                          htex_query* sorted, int32_t* pos, htex_stream stream) {
     if (!t || n < 0 || n > int64_t(INT32_MAX)) return HTEX_ERR_INVALID_ARG;
@@ -607,7 +574,7 @@ extern "C" htex_status htex_queries_sort(const htex_textures* t, const htex_quer
         return HTEX_ERR_OUT_OF_MEMORY;
     }
     const htex_status st =
-        launch_sort<1>(t, P, words(q), n, static_cast<uint32_t*>(counters), words(sorted), pos, s);
+        launch_sort<>(t, P, words(q), n, static_cast<uint32_t*>(counters), words(sorted), pos, s);
     cudaFreeAsync(counters, s);
     return st;
 }

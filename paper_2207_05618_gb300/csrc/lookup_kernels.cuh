@@ -182,11 +182,18 @@ htex_status launch_fwd(const htex_textures* t, const FwdParams& p, uint32_t flag
         }
     } else {
         auto k = t->uniform_log2n >= 0 ? k_lookup_global<DT, C, BINNED, true> : k_lookup_global<DT, C, BINNED, false>;
-        const int64_t want = (p.n + kGlobalThreads - 1) / kGlobalThreads;
         static Occupancy occupancy[2];
         const int blocks = occupancy[t->uniform_log2n >= 0].get(k, kGlobalThreads, t->device);
-        const int64_t grid = std::min<int64_t>(want, int64_t(t->num_sms) * blocks);
-        k<<<unsigned(grid), kGlobalThreads, 0, s>>>(A, p);
+        const int64_t resident = int64_t(t->num_sms) * blocks;
+        // a batch that does not fill every SM, or fills them less than twice,
+        // is spread evenly over all of them, in blocks of fewer warps: 4,096 /
+        // 40,000 / 100,000 FP32 RGB lookups 10.1 / 12.3 / 17.4 us -> 5.0 / 8.3 /
+        // 15.1 us; more rounds (300,000 and up) gain nothing from it
+        const int64_t full = resident * kGlobalThreads, rounds = p.n > full && p.n <= 2 * full ? 2 : 1;
+        const int64_t share = (p.n + resident * rounds - 1) / (resident * rounds);
+        const int threads = int(std::min<int64_t>(kGlobalThreads, (share + 31) / 32 * 32));
+        const int64_t grid = std::min<int64_t>((p.n + threads - 1) / threads, resident);
+        k<<<unsigned(grid), threads, 0, s>>>(A, p);
     }
     return cudaGetLastError() == cudaSuccess ? HTEX_OK : HTEX_ERR_CUDA;
 }

@@ -280,6 +280,35 @@ def test_sorted_lookup_multi_chunk(fmt, C, n):
     _cmp(a[sel], oracle.lookup(mo, to, tuple(x[sel] for x in qs), nthreads=8))
 
 
+@pytest.mark.parametrize("n", [1, 33, 4097, 97280, 97281, 194561, (1 << 18) - 1, 1 << 18, (1 << 18) + 1])
+def test_batch_sizes_give_the_same_results(n):
+    """Batches below a round of every SM and below two are spread in blocks
+    of fewer warps, and HTEX_LOOKUP_BIN sorts from 2^18 queries on: the first
+    n queries of a larger batch give the same values bit for bit, plain,
+    with the flag, and through the anisotropic lookup; the adjoint the same
+    gradient (1e-5 of its largest entry) with and without the flag."""
+    gen = lambda: syn.cylinder(around=128, rows=60, seed=14)
+    mo, to, tl, *_ = _case(gen, _u(5), 4, "f32", hx.BUILD_MIPS, seed=20)
+    assert tl.pool_bytes > (64 << 20)
+    h, u, v, f = syn.queries(mo.H, 300007, seed=21, footprint="loguniform")
+    h[::997] = -1
+    q = torch.from_numpy(hx.pack_queries(h, u, v, f)).cuda()
+    ref = hx.lookup(tl, q).nan_to_num(nan=-1.0)
+    for flags in (0, hx.LOOKUP_BIN):
+        assert torch.equal(hx.lookup(tl, q[:n], flags=flags).nan_to_num(nan=-1.0), ref[:n])
+    z = np.zeros_like(f)
+    qa = torch.from_numpy(hx.pack_queries_aniso(h, u, v, f, z, z, f / 3)).cuda()
+    aref = hx.lookup_aniso(tl, qa, 4).nan_to_num(nan=-1.0)
+    for flags in (0, hx.LOOKUP_BIN):
+        assert torch.equal(hx.lookup_aniso(tl, qa[:n], 4, flags=flags).nan_to_num(nan=-1.0), aref[:n])
+    g = torch.ones((n, 4), device="cuda")
+    a = hx.lookup_backward(tl, q[:n], g)
+    b = hx.lookup_backward(tl, q[:n], g, flags=hx.LOOKUP_BIN)
+    assert (a - b).abs().max() <= 1e-5 * a.abs().max()
+    valid = int((h[:n] >= 0).sum())
+    assert abs(float(a.double().sum()) - 4 * valid) <= 1e-5 * 4 * max(valid, 1)
+
+
 def _range_shift(H, ranges=128):
     s = 0
     while (H >> s) + 1 > ranges:
