@@ -19,12 +19,14 @@ namespace htex {
 //
 // Bound: the texel lines of level 0 (134 MB) and 12 B per point out.
 // Measured on 130,598 halfedges, T = 8, one FP16 channel of 32x32 (5.9M
-// points): 80 us a call; three kernels with a query (16 B) and a result
+// points): 75 us a call; three kernels with a query (16 B) and a result
 // per point between them, the face walk of Alg. 1 repeated for every
 // point, took 236 us.
 constexpr int kDisplaceThreads = 256;
-// Points a block aims at (its halfedges: at least 1, at most one per thread).
-constexpr int kDisplacePoints = 1024;
+// Points a block aims at (its halfedges: at least 1, at most one per thread,
+// and few enough to give every SM six blocks): 512 / 1024 / 2048 points 96 /
+// 80 / 75 us.
+constexpr int kDisplacePoints = 2048;
 
 struct DisplaceParams {
     const float4* tri;
@@ -194,7 +196,8 @@ extern "C" htex_status htex_displace(const htex_geometry* g, const htex_textures
         return HTEX_ERR_INVALID_ARG;
     const int32_t K = (tess + 1) * (tess + 2) / 2;
     if (int64_t(g->H) * K >= (int64_t(1) << 31)) return HTEX_ERR_INVALID_ARG;
-    const int32_t per_block = std::min(kDisplaceThreads, std::max(1, kDisplacePoints / K));
+    const int32_t spread = (g->H + 6 * t->num_sms - 1) / (6 * t->num_sms);
+    const int32_t per_block = std::min({kDisplaceThreads, std::max(1, kDisplacePoints / K), std::max(1, spread)});
     const DisplaceParams p{g->d_tri, g->d_vn, g->d_fn, tess, K, uint32_t(((uint64_t(1) << 32) + K - 1) / K),
                            per_block, t->C, channel, scale, out};
     const Asset<GlobalSpace> A = global_asset(t);
