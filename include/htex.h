@@ -246,7 +246,7 @@ void htex_textures_destroy(htex_textures* t);
  *             counting-sort the queries into ranges of consecutive halfedges first, in
  *             chunks of 2^24 queries, filter them in that order and gather
  *             the results back into query order (same results, bit for bit;
- *             scratch of 20 + 4 * channels bytes per chunk query,
+ *             scratch of about 19 + 4 * channels bytes per chunk query,
  *             allocated stream-ordered on 'stream' from a library-owned
  *             pool and released there; HTEX_ERR_OUT_OF_MEMORY when it cannot
  *             be had); HTEX_LOOKUP_GLOBAL: never stage the pool in shared

@@ -309,6 +309,33 @@ def test_batch_sizes_give_the_same_results(n):
     assert abs(float(a.double().sum()) - 4 * valid) <= 1e-5 * 4 * max(valid, 1)
 
 
+@pytest.mark.parametrize("C", [1, 2, 3, 4])
+@pytest.mark.parametrize("skew", ["one", "ends", "invalid", "sorted"])
+def test_sorted_lookup_skewed_ranges(C, skew):
+    """Tiles whose queries fall into one range, into the first and the last
+    only, into none (all invalid), or come in order (every tile a few
+    ranges), with a ragged last tile: the sorted path gives the plain one's
+    results bit for bit."""
+    gen = lambda: syn.cylinder(around=128, rows=60, seed=14)
+    mo, to, tl, *_ = _case(gen, _u(5 if C > 1 else 6), C, "u8" if C == 4 else "f32", hx.BUILD_MIPS, seed=22)
+    assert tl.pool_bytes > (64 << 20)
+    n = (1 << 18) + 2049
+    h, u, v, f = syn.queries(mo.H, n, seed=23, footprint="loguniform")
+    if skew == "one":
+        h[:] = mo.H // 2
+    elif skew == "ends":
+        h = np.where(np.arange(n) % 3 == 0, 0, mo.H - 1).astype(np.int32)
+    elif skew == "invalid":
+        h[:] = -1
+        h[n // 2] = 5
+    else:
+        h = np.sort(h)
+    q = torch.from_numpy(hx.pack_queries(h, u, v, f)).cuda()
+    a, b = hx.lookup(tl, q, flags=hx.LOOKUP_BIN), hx.lookup(tl, q)
+    assert torch.equal(torch.isnan(a), torch.isnan(b))
+    assert torch.equal(a.nan_to_num(nan=0.0), b.nan_to_num(nan=0.0))
+
+
 def _range_shift(H, ranges=128):
     s = 0
     while (H >> s) + 1 > ranges:
