@@ -386,14 +386,14 @@ __global__ void __launch_bounds__(kSortThreads) k_chunk_unsort(const float* __re
                 if (first[b + s] <= uint32_t(j)) b += s;
             const int64_t at = int64_t(from[b]) + (uint32_t(j) - first[b]);
             if constexpr (C == 4) {
-                const float4 r = __ldcs(reinterpret_cast<const float4*>(sout) + at);
+                const float4 r = __ldcg(reinterpret_cast<const float4*>(sout) + at);
                 v[k][0] = r.x; v[k][1] = r.y; v[k][2] = r.z; v[k][3] = r.w;
             } else if constexpr (C == 2) {
-                const float2 r = __ldcs(reinterpret_cast<const float2*>(sout) + at);
+                const float2 r = __ldcg(reinterpret_cast<const float2*>(sout) + at);
                 v[k][0] = r.x; v[k][1] = r.y;
             } else {
 #pragma unroll
-                for (int c = 0; c < C; ++c) v[k][c] = __ldcs(sout + at * C + c);
+                for (int c = 0; c < C; ++c) v[k][c] = __ldcg(sout + at * C + c);
             }
         }
     }
