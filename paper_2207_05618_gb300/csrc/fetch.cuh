@@ -242,6 +242,7 @@ template <int DT, int C>
 struct Raw {
     static constexpr int TB = C * Fmt<DT>::ES;
     static constexpr bool PACKED = (TB == 1 || TB == 2 || TB == 4);   // one register per texel
+    static constexpr bool DOUBLE = TB == 8;                           // two
     uint32_t a = 0u, b = 0u;
 
     template <class S>

@@ -608,7 +608,7 @@ htex_status htex_launch_lookup(const htex_textures* t, const htex_query* q, int6
     const SortRuns runs{reinterpret_cast<uint16_t*>(base + cnt_b + sq_b),
                         reinterpret_cast<uint2*>(base + cnt_b + sq_b + place_b)};
     float* sout = reinterpret_cast<float*>(base + cnt_b + sq_b + place_b + start_b);
-    const uint32_t fwd_flags = flags & ~uint32_t(HTEX_LOOKUP_BIN);
+    const uint32_t fwd_flags = (flags & ~uint32_t(HTEX_LOOKUP_BIN)) | kLookupSorted;
     htex_status st = HTEX_OK;
     for (int64_t c0 = 0; c0 < n && st == HTEX_OK; c0 += M) {
         const int64_t m = std::min<int64_t>(M, n - c0);

@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(kThreads, 5) k_raster(htex_geometry g, Camera 
         const int P = __shfl_sync(0xffffffffu, incl, 31), start = incl - mine;
         if (mine > 0) put(__popc(some & ((1u << lane) - 1u)), start);
         __syncwarp();
-        unsigned begun = 0;   // triangles that start before this round
+        unsigned begun = 0;   // triangles that start before these 32 pixels
         for (int R = 0; R < P; R += 32) {
             const unsigned starts = __reduce_or_sync(0xffffffffu,
                                                      mine > 0 && unsigned(start - R) < 32u ? 1u << (start - R) : 0u);
