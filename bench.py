@@ -906,7 +906,7 @@ def aniso_bench(hx, torch, stream, mesh, tex, n=1 << 22, reps=10, warm=3, sorted
                                                               flags=hx.LOOKUP_BIN), reps) if sorted_too else None)
     prof = profiled_values("lookup_aniso.md", ANISO_SOURCES)
     peak, _ = hbm_peak()
-    roof = {"bound": "instruction issue", "unit": "GB/s", "peak": peak}
+    roof = {"bound": "random DRAM lines", "unit": "GB/s", "peak": peak}
     if prof:
         b = prof["aniso_dram_bytes_per_lookup"]
         roof.update({"dram_bytes_per_lookup": b, "achieved": b * n / (ms / 1e3) / 1e9,
