@@ -236,7 +236,11 @@ __global__ void __launch_bounds__(kSortThreads) k_chunk_scatter(const int4* q, i
     __syncthreads();
     block_scan_buckets(cnt, start, B, warp_tot);
 
-    for (int64_t t0 = int64_t(blockIdx.x) * TILE; t0 < m; t0 += int64_t(gridDim.x) * TILE) {
+    // tiles from the chunk's end: the count pass has just read those last, and
+    // as much of them as fits is still in L2 (4M FP8 lookups 245.8 -> 243.3 us,
+    // 16M RGBA8 787 -> 784.6)
+    for (int64_t tile_no = (m - 1) / TILE - blockIdx.x; tile_no >= 0; tile_no -= gridDim.x) {
+        const int64_t t0 = tile_no * TILE;
         const int tm = int(min(int64_t(TILE), m - t0));
         for (uint32_t b = threadIdx.x; b < B; b += blockDim.x) cnt[b] = 0;
         __syncthreads();
@@ -278,7 +282,7 @@ __global__ void __launch_bounds__(kSortThreads) k_chunk_scatter(const int4* q, i
         }
         if (runs.place)
             for (uint32_t b = threadIdx.x; b < B; b += blockDim.x)
-                runs.start[(t0 / TILE) * B + b] = make_uint2(loff[b], gbase[b]);
+                runs.start[tile_no * B + b] = make_uint2(loff[b], gbase[b]);
         __syncthreads();
         for (int j = threadIdx.x; j < tm; j += kSortThreads) {
             const uint32_t b = tile_bucket[j];
