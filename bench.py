@@ -188,7 +188,7 @@ def profiled_traffic(kernel: str):
 
 
 # the files the anisotropic kernel and the adjoint are compiled from (and the build flags)
-ANISO_SOURCES = ("csrc/aniso.cu", "csrc/aniso_launch.h", "csrc/lookup_core.cuh", "csrc/fetch.cuh",
+ANISO_SOURCES = ("csrc/aniso.cu", "csrc/aniso_launch.h", "csrc/aniso_taps.h", "csrc/lookup_core.cuh", "csrc/fetch.cuh",
                  "csrc/packed.cuh", "csrc/htex_internal.h", "build.py")
 BACKWARD_SOURCES = ("csrc/backward.cu", "csrc/fetch.cuh", "csrc/htex_internal.h", "build.py")
 

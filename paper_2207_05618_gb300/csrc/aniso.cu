@@ -34,6 +34,7 @@
 
 #include "lookup_core.cuh"
 #include "aniso_launch.h"
+#include "aniso_taps.h"
 
 namespace htex {
 
@@ -43,47 +44,6 @@ struct AnisoParams {
     int32_t kmax;
     float* out;
     int32_t* status;
-};
-
-// Two taps along one axis for an arbitrary coordinate: index i = floor(s)
-// unclamped, in-bounds weights (zero for a tap outside [0, N)).
-struct TapsG {
-    int i;
-    float w0, w1;
-};
-
-__device__ __forceinline__ TapsG taps_g(float p, int N) {
-    const float s = fmaf(p, float(N), -0.5f);
-    const float fi = floorf(s);
-    const float a = s - fi;
-    const int i = int(fi);
-    return TapsG{i, (i >= 0 && i < N) ? 1.0f - a : 0.0f, (i + 1 >= 0 && i + 1 < N) ? a : 0.0f};
-}
-
-// One level of one fetch at quad coordinates (x, y): four taps, their data
-// weights (level weight and code scale included) and their loads.
-template <int DT, int C>
-struct LevelTaps {
-    static constexpr int TB = C * Fmt<DT>::ES;
-    uint64_t o;
-    uint32_t row;
-    float w[4];
-
-    // wl: the level weight; wd: the level weight times the code scale.
-    // Returns the level's share of the normalisation weight.
-    __device__ __forceinline__ float plan(uint64_t base, int n, float x, float y, float wl, float wd) {
-        const int N = 1 << n;
-        const TapsG tx = taps_g(x, N), ty = taps_g(y, N);
-        const float y0 = ty.w0 * wd, y1 = ty.w1 * wd;
-        w[0] = y0 * tx.w0;
-        w[1] = y0 * tx.w1;
-        w[2] = y1 * tx.w0;
-        w[3] = y1 * tx.w1;
-        o = base + uint64_t(int64_t(((ty.i << n) + tx.i) * TB));
-        row = uint32_t(TB) << n;
-        return wl * (tx.w0 + tx.w1) * (ty.w0 + ty.w1);
-    }
-    __device__ __forceinline__ uint64_t at(int k) const { return o + (k & 1 ? TB : 0) + (k & 2 ? row : 0u); }
 };
 
 // Shared-memory words of a query: centre u, v, the probe spacing axis (major
@@ -299,51 +259,60 @@ __global__ void __launch_bounds__(kAnisoThreads, kAnisoBlocks) k_lookup_aniso(As
             const float x = off + ((c2 & kNegX) ? -a : a), y = off + ((c2 & kNegY) ? -b : b);
 
             Sums<C> acc;
-            LevelTaps<DT, C> L0, L1;
-            float W = L0.plan(o0, n0, x, y, w0, w0 * scale);
+            LevelTaps<TB> L0, L1;
+            // The code scale: on the sums where a weighted code keeps its 24 bits
+            // (E4M3, F16: codes of at least 2^-9, 2^-24), else on each weight
+            // (BF16 codes span the FP32 range).  4M E4M3 RGBA queries of 1..16
+            // probes on 1.4 GB: 529 us on the sums, 578 us on the weights.
+            constexpr bool scale_weights = DT == HTEX_BF16, scale_sums = Fmt<DT>::SCALED && !scale_weights;
+            const auto weight = [&](const LevelTaps<TB>& L, int m) {
+                return scale_weights ? L.w[m] * scale_of(L.w[m], scale) : L.w[m];
+            };
+            float W = L0.plan(o0, n0, x, y, w0);
             const bool two = __any_sync(0xffffffffu, w1 != 0.0f);
             // the coarser level's texels follow the finer one's (its own when there is no coarser one)
             const uint64_t o1 = o0 + (uint64_t(TB) << (2 * n0));
             if constexpr (TB <= 8 && (TB & (TB - 1)) == 0 && (DT != HTEX_F32 || C == 1)) {
                 Raw<DT, C> ta[4], tb[4];   // every load before the first decode
 #pragma unroll
-                for (int m = 0; m < 4; ++m) ta[m].load_if(A.pool, L0.w[m] != 0.0f, L0.at(m), l2_leave_policy());
+                for (int m = 0; m < 4; ++m) ta[m].load_if(A.pool, L0.read(m), L0.at(m), l2_leave_policy());
                 if (two) {
-                    W += L1.plan(o1, n1, x, y, w1, w1 * scale);
+                    W += L1.plan(o1, n1, x, y, w1);
 #pragma unroll
-                    for (int m = 0; m < 4; ++m) tb[m].load_if(A.pool, L1.w[m] != 0.0f, L1.at(m), l2_leave_policy());
+                    for (int m = 0; m < 4; ++m) tb[m].load_if(A.pool, L1.read(m), L1.at(m), l2_leave_policy());
                 }
                 float v[C];
 #pragma unroll
                 for (int m = 0; m < 4; ++m) {
                     ta[m].decode(v);
-                    acc.fma(L0.w[m], v);
+                    acc.fma(weight(L0, m), v);
                 }
                 if (two) {
 #pragma unroll
                     for (int m = 0; m < 4; ++m) {
                         tb[m].decode(v);
-                        acc.fma(L1.w[m], v);
+                        acc.fma(weight(L1, m), v);
                     }
                 }
             } else {
                 float v[4][C];
 #pragma unroll
-                for (int m = 0; m < 4; ++m) load_texel_if<DT, C>(A.pool, L0.w[m] != 0.0f, L0.at(m), v[m]);
+                for (int m = 0; m < 4; ++m) load_texel_if<DT, C>(A.pool, L0.read(m), L0.at(m), v[m]);
 #pragma unroll
-                for (int m = 0; m < 4; ++m) acc.fma(L0.w[m], v[m]);
+                for (int m = 0; m < 4; ++m) acc.fma(weight(L0, m), v[m]);
                 if (two) {
-                    W += L1.plan(o1, n1, x, y, w1, w1 * scale);
+                    W += L1.plan(o1, n1, x, y, w1);
 #pragma unroll
-                    for (int m = 0; m < 4; ++m) load_texel_if<DT, C>(A.pool, L1.w[m] != 0.0f, L1.at(m), v[m]);
+                    for (int m = 0; m < 4; ++m) load_texel_if<DT, C>(A.pool, L1.read(m), L1.at(m), v[m]);
 #pragma unroll
-                    for (int m = 0; m < 4; ++m) acc.fma(L1.w[m], v[m]);
+                    for (int m = 0; m < 4; ++m) acc.fma(weight(L1, m), v[m]);
                 }
             }
             float sums[C];
             acc.get(sums);
+            const float on_sums = scale_sums ? scale_of(W, scale) : 1.0f;
 #pragma unroll
-            for (int c = 0; c < C; ++c) part[wib][lane][c] = sums[c];
+            for (int c = 0; c < C; ++c) part[wib][lane][c] = scale_sums ? sums[c] * on_sums : sums[c];
             part[wib][lane][C] = W;
             __syncwarp();
 

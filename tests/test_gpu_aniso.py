@@ -187,3 +187,32 @@ def test_aniso_probe_intervals_and_warp_mates(n):
     _cmp(got, oracle.lookup_aniso(mo, to, qs, 16), _tol(16, nmax=64))
     perm = rng.permutation(n)
     np.testing.assert_array_equal(_gpu(tl, tuple(x[perm] for x in qs), 16), got[perm])
+
+
+@pytest.mark.parametrize("fmt,C,code", [("f16", 4, 0x3800), ("f16", 1, 0x3800), ("bf16", 3, 0x3F00), ("bf16", 2, 0x3F00),
+                                        ("e4m3", 4, 0x38), ("e4m3", 3, 0x38)])
+@pytest.mark.parametrize("scale", [np.inf, -np.inf, np.nan])
+def test_aniso_scale_that_is_not_finite(fmt, C, code, scale):
+    """One texture whose code scale is infinite or NaN (an infinite texel
+    uploaded in a scaled format, or scales handed in as they are): queries
+    that weigh one of its texels are not finite, every other query has the
+    bits it has under a finite scale, whatever queries share its warp."""
+    fs, fv, V = syn.cylinder(around=12, rows=5, seed=21)[:3]
+    mesh = hx.Mesh(fs, fv, V)
+    log2n = (np.arange(mesh.E) * 5 % 7).astype(np.int32)
+    E = mesh.E // 2
+    log2n[E] = 4
+    nbytes = hx.Textures.layout(mesh, log2n, C, fmt)[0]
+    pool = np.full(nbytes // (1 if fmt == "e4m3" else 2), code, np.uint8 if fmt == "e4m3" else np.uint16).view(np.uint8)
+    qs = _aniso_queries(mesh.H, 30011, seed=5, lo=-9, hi=2)
+
+    def run(s):
+        scales = np.ones(mesh.E, np.float32)
+        scales[E] = s
+        return _gpu(hx.Textures.upload_pool(mesh, log2n, pool, scales, C, fmt), qs, 16)
+
+    base, big, got = run(1.0), run(2.0 ** 100), run(scale)
+    clean = (base == big).all(1)
+    assert 100 < clean.sum() < len(clean) - 100
+    np.testing.assert_array_equal(got[clean], base[clean])
+    assert not np.isfinite(got[~clean]).any()
