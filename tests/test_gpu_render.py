@@ -33,6 +33,18 @@ def test_triangle_vertices_match_alg1():
         np.testing.assert_allclose(got, ref, atol=2e-6)
 
 
+@pytest.mark.parametrize("around,rows", [(3, 1), (8, 7), (12, 20), (300, 260)])
+def test_triangle_vertices_block_edges(around, rows):
+    """Fewer halfedges than a block takes, a few blocks with a part of one,
+    and more than one pass of the grid (8 blocks of 256 per SM)."""
+    fs, fv, V, pos = syn.cylinder(around=around, rows=rows, seed=around)
+    mo = oracle.mesh_from_faces(fs, fv, V)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert mo.H % 256 != 0 and (mo.H > 8 * 256 * sms or around < 300)
+    got = render.Geometry(hx.Mesh(fs, fv, V), pos).triangle_vertices().cpu().numpy()
+    np.testing.assert_allclose(got, oracle.triangle_vertices(mo, pos.astype(np.float32).astype(np.float64)), atol=2e-6)
+
+
 @pytest.mark.parametrize("W,H", [(96, 64), (61, 37)])
 def test_rasterizer_matches_reference(W, H):
     """Pixels whose nearest triangle is clear (barycentric margin and depth
