@@ -398,10 +398,11 @@ htex_status htex_textures_adam_step(htex_textures* t, float* master, float* grad
  * the Htex at its (halfedge, barycentrics)), as CUDA kernels. */
 typedef struct htex_geometry htex_geometry;
 
-/* Device geometry of a mesh: its Next/Vert/Face operators, vertex
- * positions (host [V][3] float, copied) and the normals of the input mesh
- * (per face its area vector by Newell's formula, per vertex the normalised
- * sum of its faces' vectors), computed on the host.  Synchronises stream. */
+/* Device geometry of a mesh: the intrinsic triangle of every halfedge
+ * (Alg. 1, 48 bytes, evaluated here from the vertex positions, host [V][3]
+ * float) and the normals of the input mesh (per face its area vector by
+ * Newell's formula, per vertex the normalised sum of its faces' vectors),
+ * computed on the host.  Synchronises stream. */
 htex_status htex_geometry_create(const htex_mesh* m, const float* positions, htex_stream stream,
                                  htex_geometry** out);
 void htex_geometry_destroy(htex_geometry* g);
@@ -424,8 +425,10 @@ htex_status htex_triangle_vertices(const htex_geometry* g, float* out, htex_stre
  *              per pixel; h = -1 (an invalid query) where nothing is seen
  *   depth      device [height][width] float, nullable: NDC depth (NaN if empty)
  * Triangles with a vertex at or behind the camera plane (w <= 0) are not
- * drawn.  Scratch (8 bytes per pixel and 64 per halfedge) comes
- * stream-ordered from a library-owned pool.  Asynchronous. */
+ * drawn.  Scratch (8 bytes per pixel and, for meshes of no more halfedges
+ * than the frame has pixels or than 2^18, 64 per halfedge while there is
+ * memory for it) comes stream-ordered from a library-owned pool.
+ * Asynchronous. */
 htex_status htex_rasterize(const htex_geometry* g, const float* view_proj, int32_t width, int32_t height,
                            htex_query* queries, float* depth, htex_stream stream);
 

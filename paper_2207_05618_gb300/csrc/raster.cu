@@ -11,7 +11,8 @@
 // depth z/w in [-1, 1]) and the smallest 64-bit key (ordered depth << 32 |
 // halfedge) is kept per pixel with atomicMin, so ties go to the smaller
 // halfedge id.  A resolve pass turns each pixel's key into a query from the
-// projected triangle the first pass left in scratch: barycentrics at the
+// projected triangle, which the first pass left in scratch or (meshes fine
+// beside the frame) is projected again: barycentrics at the
 // pixel centre corrected for perspective, and the footprint max(|d(u,v)/dx|,
 // |d(u,v)/dy|) from the same triangle's barycentrics one pixel right and one
 // pixel down.  Triangles with a vertex behind the camera (w <= 0) are not
@@ -225,6 +226,8 @@ __device__ __forceinline__ void cover(const RasterTriangle& t, int qx, int qy, i
     atomicMin(vis + int64_t(y) * width + x, key);
 }
 
+// KEPT: the projected triangles go to 'screens'.
+template <bool KEPT>
 __global__ void __launch_bounds__(kThreads, 5) k_raster(htex_geometry g, Camera cam, unsigned long long* vis,
                                                      float4* screens) {
     __shared__ RasterTriangle tris[kThreads / 32][32];
@@ -250,7 +253,7 @@ __global__ void __launch_bounds__(kThreads, 5) k_raster(htex_geometry g, Camera 
             }
         }
         const int pixels = nx * ny;   // of the frame, which has fewer than 2^31
-        if (pixels > 0) store_screen(screens + 4 * h, s);
+        if (KEPT && pixels > 0) store_screen(screens + 4 * h, s);
         const auto put = [&](unsigned t, int first) {
             // below: 2^-140 |den|, so that the quotient is at least 2^-140
             w[t] = RasterTriangle{s.y[1] - s.y[2], s.y[2] - s.y[0], s.x[2] - s.x[1], s.x[0] - s.x[2],
@@ -302,8 +305,10 @@ __global__ void __launch_bounds__(kThreads, 5) k_raster(htex_geometry g, Camera 
 // pixel centre and at the centres one pixel right and one pixel down; Q is
 // htex_query (footprint = the longer of the two differences) or
 // htex_query_aniso (the two differences as the screen derivatives).
-template <class Q>
-__global__ void k_resolve(Camera cam, const unsigned long long* vis, const float4* screens, Q* q, float* depth) {
+// KEPT: the projected triangles are in 'screens'; otherwise projected again.
+template <class Q, bool KEPT>
+__global__ void k_resolve(htex_geometry g, Camera cam, const unsigned long long* vis, const float4* screens, Q* q,
+                          float* depth) {
     const uint32_t n = uint32_t(cam.W) * uint32_t(cam.Ht);   // below 2^31
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const unsigned long long key = vis[i];
@@ -312,7 +317,14 @@ __global__ void k_resolve(Camera cam, const unsigned long long* vis, const float
         float zd = __int_as_float(0x7fc00000);
         if (key != ~0ull) {
             h = int32_t(uint32_t(key & 0xffffffffull));
-            const Screen s = load_screen(screens + 4 * int64_t(h));
+            Screen s;
+            if constexpr (KEPT) {
+                s = load_screen(screens + 4 * int64_t(h));
+            } else {
+                float3 v[3];
+                triangle(g, h, v[0], v[1], v[2]);
+                project(cam, v, s);
+            }
             const uint32_t row = i / uint32_t(cam.W);
             const float px = float(i - row * uint32_t(cam.W)) + 0.5f, py = float(row) + 0.5f;
             float ux, vx, uy, vy;
@@ -473,17 +485,30 @@ htex_status rasterize(const htex_geometry* g, const float* view_proj, int32_t wi
     if (cudaGetDevice(&dev) != cudaSuccess) return HTEX_ERR_CUDA;
     cudaMemPool_t pool = work_pool(dev);
     if (!pool) return HTEX_ERR_CUDA;
-    void* vis = nullptr;   // the pixels' keys, then the projected triangles
+    // The pixels' keys, then the projected triangles where they are kept: for
+    // meshes of at most as many halfedges as the frame has pixels, or 2^18 (so
+    // that this scratch stays within 64 bytes a pixel or 16 MiB), and while
+    // there is memory for them.  Kept / projected again, halfedges per pixel
+    // 0.06: 218 / 238 us, 0.25: 68 / 74, 0.57: 42 / 45 and 69 / 66, 1.3: 48 /
+    // 45, 2.2: 129 / 127; 14,400 pixels of 57k halfedges 14.4 / 16.4.
     const size_t vis_b = (size_t(n) * 8 + 63) & ~size_t(63);
-    if (cudaMallocFromPoolAsync(&vis, vis_b + size_t(g->H) * 64, pool, s) != cudaSuccess) {
+    void* vis = nullptr;
+    bool kept = g->H <= std::max<int64_t>(n, int64_t(1) << 18);
+    kept = kept && cudaMallocFromPoolAsync(&vis, vis_b + size_t(g->H) * 64, pool, s) == cudaSuccess;
+    if (!kept) {
         cudaGetLastError();
-        return HTEX_ERR_OUT_OF_MEMORY;
+        if (cudaMallocFromPoolAsync(&vis, vis_b, pool, s) != cudaSuccess) {
+            cudaGetLastError();
+            return HTEX_ERR_OUT_OF_MEMORY;
+        }
     }
     auto* v = static_cast<unsigned long long*>(vis);
-    auto* screens = reinterpret_cast<float4*>(static_cast<uint8_t*>(vis) + vis_b);
+    auto* screens = kept ? reinterpret_cast<float4*>(static_cast<uint8_t*>(vis) + vis_b) : nullptr;
     k_clear<<<grid_for(int64_t(vis_b / 16)), kThreads, 0, s>>>(static_cast<ulonglong2*>(vis), int64_t(vis_b / 16));
-    k_raster<<<grid_for(g->H), kThreads, 0, s>>>(*g, cam, v, screens);
-    k_resolve<Q><<<grid_for(n), kThreads, 0, s>>>(cam, v, screens, queries, depth);
+    const auto raster = kept ? k_raster<true> : k_raster<false>;
+    const auto resolve = kept ? k_resolve<Q, true> : k_resolve<Q, false>;
+    raster<<<grid_for(g->H), kThreads, 0, s>>>(*g, cam, v, screens);
+    resolve<<<grid_for(n), kThreads, 0, s>>>(*g, cam, v, screens, queries, depth);
     const bool ok = cudaGetLastError() == cudaSuccess;
     cudaFreeAsync(vis, s);
     return ok ? HTEX_OK : HTEX_ERR_CUDA;

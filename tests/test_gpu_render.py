@@ -195,3 +195,27 @@ def test_rasterizer_small_and_large_boxes(W, H, eye):
     np.testing.assert_allclose(depth.cpu().numpy().reshape(H, W)[clear], dref[clear], atol=1e-5)
     empty = gh < 0
     assert np.all((hh[empty] < 0) | (margin[empty] < 1e-3))
+
+
+@pytest.mark.parametrize("aniso", [False, True])
+def test_rasterizer_projected_triangles_kept_or_not(aniso):
+    """A small mesh (whose projected triangles are kept between the passes),
+    and the same mesh with faces behind the camera added until it has more
+    than 2^18 halfedges and than the frame has pixels (projected again): the
+    same queries and depths, bit for bit."""
+    W, H = 96, 64
+    fs, fv, V, pos = _sphere()
+    M = syn.perspective(40.0, W / H, 0.3, 10.0) @ syn.look_at([2.3, -1.1, 0.9], [0, 0, 0], [0, 0, 1])
+    fs2, fv2, V2, pos2 = syn.cylinder(around=300, rows=260, seed=1)
+    more = (np.concatenate([fs, fs2]), np.concatenate([fv, fv2 + V]), V + V2,
+            np.concatenate([pos, pos2 * 0.2 + [4.6, -2.2, 1.8]]))
+    got = []
+    for f, v, n, p in ((fs, fv, V, pos), more):
+        g = render.Geometry(hx.Mesh(f, v, n), p)
+        depth = torch.empty(W * H, dtype=torch.float32, device="cuda")
+        q = (g.rasterize_aniso if aniso else g.rasterize)(M, W, H, depth=depth)
+        got.append((g.H, q.cpu().numpy(), depth.cpu().numpy().view(np.int32)))
+    assert got[0][0] < W * H < 1 << 18 < got[1][0]
+    assert (got[0][1][:, 0] >= 0).mean() > 0.1
+    np.testing.assert_array_equal(got[0][1], got[1][1])
+    np.testing.assert_array_equal(got[0][2], got[1][2])
