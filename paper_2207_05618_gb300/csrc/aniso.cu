@@ -98,12 +98,18 @@ __device__ __forceinline__ int aniso_probes(float px2, float py2, int kmax) {
 
 constexpr int kAnisoThreads = 128;
 constexpr int kAnisoWarps = kAnisoThreads / 32;
-// Resident blocks per SM (56 registers a thread).  The kernel is bound by
-// random 128-byte lines from DRAM and their latency: 4M queries of 1..16
-// probes on a 1.4 GB RGBA8 asset take 582 / 538 / 551 / 586 us at 8 / 9 /
-// 10 / 11 blocks (2.8 GB of lines, 5.2 TB/s at 9; independent random lines
-// reach 5.2 TB/s).
-constexpr int kAnisoBlocks = 9;
+// Resident blocks per SM.  The kernel is bound by random 128-byte lines from
+// DRAM and their latency: 4M queries of 1..16 probes on a 1.4 GB RGBA8 asset
+// take 569 / 517 / 546 us at 8 / 9 / 10 blocks (2.8 GB of lines, 5.2 TB/s at
+// 9; independent random lines reach 5.2 TB/s).  At 9 a thread has 56
+// registers, and the one-, two- and four-channel kernels spill 4 to 20 bytes.
+// FP32 RG and RGBA texels want fewer: with at most two probes a query (few
+// shared lines) 385 / 323 / 340 and 497 / 417 / 390 us at 9 / 8 / 7, with 16
+// probes 567 / 561 / 599 and 666 / 675 / 668.
+template <int DT, int C>
+constexpr int aniso_blocks() {
+    return DT != HTEX_F32 ? 9 : C == 4 ? 7 : C == 2 ? 8 : 9;
+}
 
 // A decoded anisotropic query: validity, the probe count and line, and the
 // footprint of one probe.
@@ -136,8 +142,8 @@ __device__ __forceinline__ AnisoQuery decode_aniso(int4 r0, int4 r1, int32_t H, 
 // SPREAD: a warp takes 'few' queries at a time instead of 32 (small batches;
 // as a variant of its own, since the run-time count costs the full batches 8%).
 template <int DT, int C, bool SPREAD>
-__global__ void __launch_bounds__(kAnisoThreads, kAnisoBlocks) k_lookup_aniso(Asset<GlobalSpace> A, AnisoParams p,
-                                                                              int few) {
+__global__ void __launch_bounds__(kAnisoThreads, (aniso_blocks<DT, C>()))
+k_lookup_aniso(Asset<GlobalSpace> A, AnisoParams p, int few) {
     constexpr int TB = C * Fmt<DT>::ES;
     constexpr int FW = Fmt<DT>::SCALED ? 5 : 4;      // words per fetch
     __shared__ uint32_t consts[kAnisoWarps][kFetch + 3 * FW][32];
