@@ -278,10 +278,13 @@ htex_status htex_lookup(const htex_textures* t, const htex_query* q, int64_t n, 
  *   placed.
  *   q          device [n] htex_query_aniso (16-byte aligned)
  *   max_aniso  1..16
- *   flags      HTEX_LOOKUP_BIN: accepted; the queries are filtered in their
- *              given order all the same (results never depend on the
- *              order: each query's probes are summed in an order of its
- *              own; sorting was slower at every size)
+ *   flags      HTEX_LOOKUP_BIN: with max_aniso = 1, texels of 6 bytes or
+ *              more, 2^21 queries or more and a pool above 64 MiB, sort the
+ *              queries as htex_lookup does (scratch of about 35 + 4 *
+ *              channels bytes per chunk query); else they are filtered in
+ *              their given order, which is faster.  The same results
+ *              either way, bit for bit: each query's probes are summed in
+ *              an order of its own
  *   out        device [n][channels] float (alignment as htex_lookup)
  *   d_status   device int32, nullable: incremented once per invalid query
  *              (h out of range, non-finite u, v or derivative, or an

@@ -265,7 +265,7 @@ def pack_queries_aniso(h, u, v, dudx, dvdx, dudy, dvdy) -> np.ndarray:
 
 def lookup_aniso(tex: Textures, queries, max_aniso: int = 16, out=None, stream=None, status=None, flags: int = 0):
     """htex_lookup_aniso: queries int32 CUDA tensor [n, 8] -> float32 [n, channels]
-    (flags: LOOKUP_BIN is accepted and changes nothing)."""
+    (flags: LOOKUP_BIN sorts large batches of one probe a query; the same results)."""
     import torch
     _check_tensor(queries, "queries", torch.int32, 8)
     n = queries.shape[0]

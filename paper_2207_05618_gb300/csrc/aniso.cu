@@ -413,9 +413,6 @@ extern "C" htex_status htex_lookup_aniso(const htex_textures* t, const htex_quer
     if ((reinterpret_cast<uintptr_t>(q) & 15u) != 0) return HTEX_ERR_INVALID_ARG;
     const uintptr_t out_align = t->C == 4 ? 16u : (t->C == 2 ? 8u : 4u);
     if ((reinterpret_cast<uintptr_t>(out) & (out_align - 1)) != 0) return HTEX_ERR_INVALID_ARG;
-    // HTEX_LOOKUP_BIN is accepted, and the queries filtered as they come: a query
-    // spends its time on its own probes' lines, of which few are shared, and
-    // sorting 32-byte queries never paid (1M / 4M / 16M random queries, 1.4 GB
-    // RGBA8: 136 / 518 / 1992 us as they come, 180 / 636 / 2438 us sorted)
+    if (flags & HTEX_LOOKUP_BIN) return htex_launch_aniso_sorted(t, q, n, max_aniso, out, stream, d_status);
     return htex_launch_aniso(t, q, n, max_aniso, out, stream, d_status);
 }

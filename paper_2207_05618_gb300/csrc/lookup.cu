@@ -30,6 +30,7 @@
 #include <cuda_runtime.h>
 
 #include "lookup_kernels.cuh"
+#include "aniso_launch.h"
 
 namespace htex {
 
@@ -128,8 +129,8 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_scatter(const htex_query* q
 // ------------------------------------------ chunk-local sort (HTEX_LOOKUP_BIN)
 //
 // One chunk of m queries at a time: a bucket histogram, then per tile of
-// kSortThreads x kSortPer queries (half as many per thread with a payload)
-// a local counting sort in shared memory, so that every
+// kSortThreads x kSortPer queries (fewer per thread for wider queries or a
+// payload) a local counting sort in shared memory, so that every
 // bucket's run of the tile is written to the sorted copy as one contiguous
 // piece (whole sectors, not scattered 16-byte pieces), and each query's
 // sorted position is recorded in query order.  The lookup then filters the
@@ -141,9 +142,12 @@ constexpr int kSortThreads = 256;
 constexpr int kSortPer = 8;   // 16-byte query words per thread and tile (16: 8% slower sort, measured)
 constexpr int kSortMaxBuckets = 256;
 
+// QW: 16-byte words per query (1: htex_query, 2: htex_query_aniso); the
+// halfedge id is the first word's first int.
+template <int QW>
 __global__ void __launch_bounds__(kSortThreads) k_chunk_count(const int4* q, int64_t m, int32_t H, int shift,
                                                               uint32_t B, uint32_t* counts) {
-    constexpr int PER = kSortPer, TILE = kSortThreads * PER;
+    constexpr int PER = kSortPer / QW, TILE = kSortThreads * PER;
     __shared__ uint32_t hist[kSortMaxBuckets];
     for (uint32_t b = threadIdx.x; b < B; b += blockDim.x) hist[b] = 0;
     __syncthreads();
@@ -152,7 +156,7 @@ __global__ void __launch_bounds__(kSortThreads) k_chunk_count(const int4* q, int
 #pragma unroll
         for (int k = 0; k < PER; ++k) {
             const int64_t i = t0 + int64_t(k) * kSortThreads + threadIdx.x;
-            h[k] = i < m ? __ldg(reinterpret_cast<const int32_t*>(q + i)) : 0;
+            h[k] = i < m ? __ldg(reinterpret_cast<const int32_t*>(q + i * QW)) : 0;
         }
 #pragma unroll
         for (int k = 0; k < PER; ++k)
@@ -199,15 +203,14 @@ struct SortRuns {
 
 // PC: floats of payload per query (rows of 'pay' in query order, moved to
 // 'spay' in sorted order with their queries); pos nullable.
-// Shared memory of k_chunk_scatter<PC> (dynamic: a tile can exceed the
-// 48 KiB of static shared memory): the tile's queries and payload rows,
-// their buckets, and per bucket the first sorted position,
-// the tile's count, local offset and global base.
-template <int PC>
+// Shared memory of k_chunk_scatter<QW, PC> (dynamic): the tile's queries (QW
+// words each) and payload rows, their buckets, and per bucket the first
+// sorted position, the tile's count, local offset and global base.
+template <int QW, int PC>
 struct ScatterSmem {
-    static constexpr int PER = kSortPer / (PC > 0 ? 2 : 1), TILE = kSortThreads * PER;
+    static constexpr int PER = kSortPer / QW / (PC > 0 ? 2 : 1), TILE = kSortThreads * PER;
     static constexpr size_t tile = 0;
-    static constexpr size_t pay = tile + size_t(TILE) * 16;
+    static constexpr size_t pay = tile + size_t(TILE) * QW * 16;
     static constexpr size_t bucket = pay + ((size_t(PC > 0 ? TILE * PC : 1) * 4 + 15) & ~size_t(15));
     static constexpr size_t arrays = bucket + ((size_t(TILE) * 2 + 15) & ~size_t(15));
     static constexpr size_t warps = arrays + size_t(4) * kSortMaxBuckets * 4;
@@ -216,12 +219,12 @@ struct ScatterSmem {
 
 // runs: nullable; where each tile's runs went and each query's place in its
 // sorted tile, for k_chunk_unsort (instead of pos).
-template <int PC>
+template <int QW, int PC>
 __global__ void __launch_bounds__(kSortThreads) k_chunk_scatter(const int4* q, int64_t m, int32_t H, int shift,
                                                                 uint32_t B, const uint32_t* counts, uint32_t* taken,
                                                                 int4* sq, int32_t* pos, int32_t pos_base,
                                                                 const float* pay, float* spay, SortRuns runs) {
-    using L = ScatterSmem<PC>;
+    using L = ScatterSmem<QW, PC>;
     constexpr int PER = L::PER, TILE = L::TILE;
     extern __shared__ __align__(16) uint8_t smem[];
     int4* tile = reinterpret_cast<int4*>(smem + L::tile);
@@ -244,13 +247,15 @@ __global__ void __launch_bounds__(kSortThreads) k_chunk_scatter(const int4* q, i
         const int tm = int(min(int64_t(TILE), m - t0));
         for (uint32_t b = threadIdx.x; b < B; b += blockDim.x) cnt[b] = 0;
         __syncthreads();
-        int4 r[PER];
+        int4 r[PER][QW];
         float pv[PER][PC > 0 ? PC : 1];
         uint32_t bk[PER], rank[PER];
 #pragma unroll
         for (int k = 0; k < PER; ++k) {
             const int j = k * kSortThreads + threadIdx.x;
-            if (j < tm) r[k] = __ldcs(q + t0 + j);
+#pragma unroll
+            for (int w = 0; w < QW; ++w)
+                if (j < tm) r[k][w] = __ldcs(q + (t0 + j) * QW + w);
 #pragma unroll
             for (int c = 0; c < PC; ++c)
                 if (j < tm) pv[k][c] = __ldcs(pay + (t0 + j) * PC + c);
@@ -258,7 +263,7 @@ __global__ void __launch_bounds__(kSortThreads) k_chunk_scatter(const int4* q, i
 #pragma unroll
         for (int k = 0; k < PER; ++k) {
             if (k * kSortThreads + int(threadIdx.x) < tm) {
-                bk[k] = bucket_of(r[k].x, H, shift, B - 1);
+                bk[k] = bucket_of(r[k][0].x, H, shift, B - 1);
                 rank[k] = atomicAdd(&cnt[bk[k]], 1u);
             }
         }
@@ -272,7 +277,8 @@ __global__ void __launch_bounds__(kSortThreads) k_chunk_scatter(const int4* q, i
             const int j = k * kSortThreads + threadIdx.x;
             if (j < tm) {
                 const uint32_t lp = loff[bk[k]] + rank[k];
-                tile[lp] = r[k];
+#pragma unroll
+                for (int w = 0; w < QW; ++w) tile[lp * QW + w] = r[k][w];
 #pragma unroll
                 for (int c = 0; c < PC; ++c) tile_pay[lp * PC + c] = pv[k][c];
                 tile_bucket[lp] = uint16_t(bk[k]);
@@ -284,9 +290,10 @@ __global__ void __launch_bounds__(kSortThreads) k_chunk_scatter(const int4* q, i
             for (uint32_t b = threadIdx.x; b < B; b += blockDim.x)
                 runs.start[tile_no * B + b] = make_uint2(loff[b], gbase[b]);
         __syncthreads();
-        for (int j = threadIdx.x; j < tm; j += kSortThreads) {
+        for (int x = threadIdx.x; x < tm * QW; x += kSortThreads) {   // one 16-byte word per thread
+            const int j = x / QW, w = x - j * QW;
             const uint32_t b = tile_bucket[j];
-            sq[gbase[b] + (uint32_t(j) - loff[b])] = tile[j];
+            sq[int64_t(gbase[b] + (uint32_t(j) - loff[b])) * QW + w] = tile[x];
         }
         if constexpr (PC > 0) {
             for (int x = threadIdx.x; x < tm * PC; x += kSortThreads) {
@@ -358,18 +365,18 @@ __global__ void k_chunk_gather(const float* __restrict__ sout, const int32_t* __
 // memory in the tile's sorted order, and written out in query order.  16M
 // RGBA results: 97 us (5.9 TB/s of its 34 B a row) against 136 us by
 // k_chunk_gather with four bytes of position a row.
-template <int C>
+template <int C, int PER>
 __global__ void __launch_bounds__(kSortThreads) k_chunk_unsort(const float* __restrict__ sout, SortRuns runs, int64_t m,
                                                                uint32_t B, float* __restrict__ out) {
-    constexpr int TILE = kSortThreads * kSortPer;
+    constexpr int TILE = kSortThreads * PER;
     extern __shared__ __align__(16) float rows[];           // [TILE][C]
     __shared__ uint32_t first[kSortMaxBuckets];             // the runs' first places in the tile, ascending
     __shared__ uint32_t from[kSortMaxBuckets];
     const int64_t t0 = int64_t(blockIdx.x) * TILE;
     const int tm = int(min(int64_t(TILE), m - t0));
-    uint32_t place[kSortPer];
+    uint32_t place[PER];
 #pragma unroll
-    for (int k = 0; k < kSortPer; ++k) {
+    for (int k = 0; k < PER; ++k) {
         const int j = k * kSortThreads + threadIdx.x;
         place[k] = j < tm ? __ldcs(runs.place + t0 + j) : 0;
     }
@@ -379,9 +386,9 @@ __global__ void __launch_bounds__(kSortThreads) k_chunk_unsort(const float* __re
         from[b] = r.y;
     }
     __syncthreads();
-    float v[kSortPer][C];
+    float v[PER][C];
 #pragma unroll
-    for (int k = 0; k < kSortPer; ++k) {
+    for (int k = 0; k < PER; ++k) {
         const int j = k * kSortThreads + threadIdx.x;
         if (j < tm) {
             uint32_t b = 0;   // the last run that starts at or before j: empty runs start where the next one does
@@ -402,7 +409,7 @@ __global__ void __launch_bounds__(kSortThreads) k_chunk_unsort(const float* __re
         }
     }
 #pragma unroll
-    for (int k = 0; k < kSortPer; ++k) {
+    for (int k = 0; k < PER; ++k) {
         const int j = k * kSortThreads + threadIdx.x;
         if (j < tm) {
             if constexpr (C == 4) reinterpret_cast<float4*>(rows)[j] = make_float4(v[k][0], v[k][1], v[k][2], v[k][3]);
@@ -415,7 +422,7 @@ __global__ void __launch_bounds__(kSortThreads) k_chunk_unsort(const float* __re
     }
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < kSortPer; ++k) {
+    for (int k = 0; k < PER; ++k) {
         const int j = k * kSortThreads + threadIdx.x;
         if (j >= tm) break;
         if constexpr (C == 4) {
@@ -453,6 +460,23 @@ constexpr int64_t kBucketTexelBytes = int64_t(32) << 20;
 // 1M: 82 / 91); the adjoint 24 / 31 / 49 and 8 / 27 / 43 us.
 constexpr int64_t kMinSortedQueries = int64_t(1) << 18;
 
+// When HTEX_LOOKUP_BIN sorts anisotropic queries: of one probe each, texels
+// of 6 bytes or more, 2^21 queries or more.  Several probes spend their time
+// on lines that few queries share; sorting 32-byte queries costs more.
+// Random queries as they come / sorted, us (130k halfedges, 64x64 texels, 0.36
+// to 5.7 GB):
+//                    one probe                       2 probes   16 probes
+//               1M         4M         16M            4M         4M
+//   FP32 RGBA   105 / 123  390 / 377  1524 / 1408    401 / 448  678 / 708
+//   FP32 RGB    130 / 121  496 / 375  1953 / 1376    449 / 453  667 / 712
+//   FP16 RGBA   107 / 115  401 / 366  1575 / 1380    365 / 423  583 / 636
+//   FP16 RGB    114 / 124  434 / 387  1708 / 1435    425 / 462  675 / 712
+//   E4M3 RGBA    91 / 106  335 / 360  1305 / 1366    344 / 419  531 / 641
+//   RGBA8        85 / 103  308 / 351  1191 / 1332    313 / 408  518 / 628
+//   one E4M3     58 /  94  212 / 305   823 / 1166    252 / 351  466 / 561
+constexpr int64_t kMinSortedAniso = int64_t(1) << 21;
+constexpr int kMinSortedAnisoTexel = 6;
+
 template <bool BINNED>
 htex_status launch_fwd_dt(const htex_textures* t, const FwdParams& p, uint32_t flags, cudaStream_t s) {
     switch (t->dtype) {
@@ -485,10 +509,6 @@ cudaMemPool_t htex_scratch_pool(int device) {
     }
     return pools[device];
 }
-
-namespace {
-
-}  // namespace
 
 // Halfedges per bucket (log2) so one bucket's textures take about
 // kBucketTexelBytes; returns -1 when the asset is too small to gain.
@@ -523,23 +543,23 @@ size_t counter_bytes(const SortPlan& P) { return (size_t(2 * P.B) * 4 + 255) & ~
 // pos[i] = where query i went (nullable); PC floats of payload per query
 // follow their queries from pay to spay; runs (at most one chunk): see
 // SortRuns.  counters: counter_bytes(P) of scratch.
-template <int PC = 0>
+template <int QW, int PC = 0>
 htex_status launch_sort(const htex_textures* t, const SortPlan& P, const int4* q, int64_t m, uint32_t* counters,
                         int4* sq, int32_t* pos, cudaStream_t s, const float* pay = nullptr, float* spay = nullptr,
                         SortRuns runs = {}) {
-    constexpr int64_t TILE = ScatterSmem<PC>::TILE;
-    constexpr size_t smem = ScatterSmem<PC>::bytes;
+    constexpr int64_t TILE = ScatterSmem<QW, PC>::TILE;
+    constexpr size_t smem = ScatterSmem<QW, PC>::bytes;
     static Occupancy occupancy;
-    const int resident = occupancy.get(k_chunk_scatter<PC>, kSortThreads, t->device, smem);
+    const int resident = occupancy.get(k_chunk_scatter<QW, PC>, kSortThreads, t->device, smem);
     if (resident == 0) return HTEX_ERR_CUDA;
     const int64_t blocks = int64_t(t->num_sms) * resident;
     for (int64_t c0 = 0; c0 < m; c0 += kSortChunk) {
         const int64_t mc = std::min<int64_t>(kSortChunk, m - c0);
         const int64_t g = std::min<int64_t>((mc + TILE - 1) / TILE, blocks);
         if (cudaMemsetAsync(counters, 0, size_t(2 * P.B) * 4, s) != cudaSuccess) return HTEX_ERR_CUDA;
-        k_chunk_count<<<unsigned(g), kSortThreads, 0, s>>>(q + c0, mc, t->H, P.shift, P.B, counters);
-        k_chunk_scatter<PC><<<unsigned(g), kSortThreads, smem, s>>>(
-            q + c0, mc, t->H, P.shift, P.B, counters, counters + P.B, sq + c0, pos ? pos + c0 : nullptr,
+        k_chunk_count<QW><<<unsigned(g), kSortThreads, 0, s>>>(q + c0 * QW, mc, t->H, P.shift, P.B, counters);
+        k_chunk_scatter<QW, PC><<<unsigned(g), kSortThreads, smem, s>>>(
+            q + c0 * QW, mc, t->H, P.shift, P.B, counters, counters + P.B, sq + c0 * QW, pos ? pos + c0 : nullptr,
             int32_t(c0), PC ? pay + c0 * PC : nullptr, PC ? spay + c0 * PC : nullptr, runs);
         if (cudaGetLastError() != cudaSuccess) return HTEX_ERR_CUDA;
     }
@@ -566,38 +586,35 @@ htex_status launch_gather(const float* sout, const int32_t* pos, int64_t m, int 
 }
 
 // The same for one chunk sorted with SortRuns.
+template <int QW>
 htex_status launch_unsort(const float* sout, const SortRuns& runs, int64_t m, uint32_t B, int C, float* out,
                           cudaStream_t s) {
-    const int64_t tile = ScatterSmem<0>::TILE;
+    constexpr int PER = ScatterSmem<QW, 0>::PER;
+    const int64_t tile = ScatterSmem<QW, 0>::TILE;
     const unsigned g = unsigned((m + tile - 1) / tile);
     const size_t smem = size_t(tile) * 4 * size_t(C);   // at most 32 KiB
     switch (C) {
-    case 1: k_chunk_unsort<1><<<g, kSortThreads, smem, s>>>(sout, runs, m, B, out); break;
-    case 2: k_chunk_unsort<2><<<g, kSortThreads, smem, s>>>(sout, runs, m, B, out); break;
-    case 3: k_chunk_unsort<3><<<g, kSortThreads, smem, s>>>(sout, runs, m, B, out); break;
-    case 4: k_chunk_unsort<4><<<g, kSortThreads, smem, s>>>(sout, runs, m, B, out); break;
+    case 1: k_chunk_unsort<1, PER><<<g, kSortThreads, smem, s>>>(sout, runs, m, B, out); break;
+    case 2: k_chunk_unsort<2, PER><<<g, kSortThreads, smem, s>>>(sout, runs, m, B, out); break;
+    case 3: k_chunk_unsort<3, PER><<<g, kSortThreads, smem, s>>>(sout, runs, m, B, out); break;
+    case 4: k_chunk_unsort<4, PER><<<g, kSortThreads, smem, s>>>(sout, runs, m, B, out); break;
     default: return HTEX_ERR_INVALID_ARG;
     }
     return cudaGetLastError() == cudaSuccess ? HTEX_OK : HTEX_ERR_CUDA;
 }
 
-}  // namespace
-
-htex_status htex_launch_lookup(const htex_textures* t, const htex_query* q, int64_t n, float* out,
-                               uint32_t flags, htex_stream stream, int32_t* d_status) {
-    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    if (!(flags & HTEX_LOOKUP_BIN) || htex_bin_shift(t) < 0 || n < kMinSortedQueries)
-        return launch_fwd_dt<false>(t, FwdParams{q, n, out, d_status, nullptr}, flags, s);
-
-    // one chunk at a time: sort, filter into the sorted copy, un-sort
-    // (storing each result straight to its query's row from the filter
-    // instead was measured slower: scattered 16-byte stores leave partly
-    // written sectors that DRAM has to merge)
+// One chunk at a time: sort, filter into the sorted copy, un-sort (storing
+// each result straight to its query's row from the filter instead was
+// measured slower: scattered 16-byte stores leave partly written sectors
+// that DRAM has to merge).  filter(sorted queries, their number, results).
+template <int QW, class Filter>
+htex_status lookup_sorted(const htex_textures* t, const int4* q, int64_t n, float* out, cudaStream_t s,
+                          const Filter& filter) {
     const SortPlan P = sort_plan(t->H);
     const int64_t M = std::min<int64_t>(n, kSortChunk);
     const size_t cnt_b = counter_bytes(P);
-    const size_t tiles = size_t((M + ScatterSmem<0>::TILE - 1) / ScatterSmem<0>::TILE);
-    const size_t sq_b = size_t(M) * 16, place_b = (size_t(M) * 2 + 255) & ~size_t(255);
+    const size_t tiles = size_t((M + ScatterSmem<QW, 0>::TILE - 1) / ScatterSmem<QW, 0>::TILE);
+    const size_t sq_b = size_t(M) * 16 * QW, place_b = (size_t(M) * 2 + 255) & ~size_t(255);
     const size_t start_b = (tiles * P.B * 8 + 255) & ~size_t(255), sout_b = size_t(M) * 4 * size_t(t->C);
     cudaMemPool_t pool = htex_scratch_pool(t->device);
     if (!pool) return HTEX_ERR_CUDA;
@@ -608,26 +625,51 @@ htex_status htex_launch_lookup(const htex_textures* t, const htex_query* q, int6
     }
     uint8_t* base = static_cast<uint8_t*>(scratch);
     uint32_t* counters = reinterpret_cast<uint32_t*>(base);
-    htex_query* sq = reinterpret_cast<htex_query*>(base + cnt_b);
+    int4* sq = reinterpret_cast<int4*>(base + cnt_b);
     const SortRuns runs{reinterpret_cast<uint16_t*>(base + cnt_b + sq_b),
                         reinterpret_cast<uint2*>(base + cnt_b + sq_b + place_b)};
     float* sout = reinterpret_cast<float*>(base + cnt_b + sq_b + place_b + start_b);
-    const uint32_t fwd_flags = (flags & ~uint32_t(HTEX_LOOKUP_BIN)) | kLookupSorted;
     htex_status st = HTEX_OK;
     for (int64_t c0 = 0; c0 < n && st == HTEX_OK; c0 += M) {
         const int64_t m = std::min<int64_t>(M, n - c0);
-        st = launch_sort<>(t, P, words(q + c0), m, counters, words(sq), nullptr, s, nullptr, nullptr, runs);
-        if (st == HTEX_OK) st = launch_fwd_dt<false>(t, FwdParams{sq, m, sout, d_status, nullptr}, fwd_flags, s);
-        if (st == HTEX_OK) st = launch_unsort(sout, runs, m, P.B, t->C, out + c0 * t->C, s);
+        st = launch_sort<QW>(t, P, q + c0 * QW, m, counters, sq, nullptr, s, nullptr, nullptr, runs);
+        if (st == HTEX_OK) st = filter(sq, m, sout);
+        if (st == HTEX_OK) st = launch_unsort<QW>(sout, runs, m, P.B, t->C, out + c0 * t->C, s);
     }
     cudaFreeAsync(scratch, s);
     return st;
 }
 
+}  // namespace
+
+htex_status htex_launch_lookup(const htex_textures* t, const htex_query* q, int64_t n, float* out,
+                               uint32_t flags, htex_stream stream, int32_t* d_status) {
+    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    if (!(flags & HTEX_LOOKUP_BIN) || htex_bin_shift(t) < 0 || n < kMinSortedQueries)
+        return launch_fwd_dt<false>(t, FwdParams{q, n, out, d_status, nullptr}, flags, s);
+
+    const uint32_t fwd_flags = (flags & ~uint32_t(HTEX_LOOKUP_BIN)) | kLookupSorted;
+    return lookup_sorted<1>(t, words(q), n, out, s, [&](const int4* sq, int64_t m, float* sout) {
+        return launch_fwd_dt<false>(t, FwdParams{reinterpret_cast<const htex_query*>(sq), m, sout, d_status, nullptr},
+                                    fwd_flags, s);
+    });
+}
+
+htex_status htex_launch_aniso_sorted(const htex_textures* t, const htex_query_aniso* q, int64_t n, int32_t kmax,
+                                     float* out, htex_stream stream, int32_t* d_status) {
+    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    if (htex_bin_shift(t) < 0 || kmax > 1 || n < kMinSortedAniso ||
+        t->C * htex_elem_size(t->dtype) < kMinSortedAnisoTexel)
+        return htex_launch_aniso(t, q, n, kmax, out, stream, d_status);
+    return lookup_sorted<2>(t, reinterpret_cast<const int4*>(q), n, out, s, [&](const int4* sq, int64_t m, float* sout) {
+        return htex_launch_aniso(t, reinterpret_cast<const htex_query_aniso*>(sq), m, kmax, sout, stream, d_status);
+    });
+}
+
 template <int C>
 htex_status launch_sort_rows(const htex_textures* t, const SortPlan& P, const htex_query* q, int64_t m,
                              const float* g, uint32_t* counters, htex_query* sq, float* sg, cudaStream_t s) {
-    return launch_sort<C>(t, P, words(q), m, counters, words(sq), nullptr, s, g, sg);
+    return launch_sort<1, C>(t, P, words(q), m, counters, words(sq), nullptr, s, g, sg);
 }
 
 // The adjoint on sorted queries: each chunk sorted by halfedge range with
@@ -690,7 +732,7 @@ extern "C" htex_status htex_queries_sort(const htex_textures* t, const htex_quer
         return HTEX_ERR_OUT_OF_MEMORY;
     }
     const htex_status st =
-        launch_sort<>(t, P, words(q), n, static_cast<uint32_t*>(counters), words(sorted), pos, s);
+        launch_sort<1>(t, P, words(q), n, static_cast<uint32_t*>(counters), words(sorted), pos, s);
     cudaFreeAsync(counters, s);
     return st;
 }

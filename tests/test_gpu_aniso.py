@@ -132,10 +132,10 @@ def test_aniso_invalid_queries_and_arguments():
 
 
 def test_sorted_aniso_equals_unsorted_multi_chunk():
-    """HTEX_LOOKUP_BIN on the anisotropic lookup: 32-byte queries sorted by
-    halfedge range in chunks of 2^24 (a full chunk and a ragged one, invalid
-    queries inside) on a pool above the 64 MiB threshold give the unsorted
-    results bit for bit, and the oracle's on a sample."""
+    """HTEX_LOOKUP_BIN with 16 probes on a pool above the 64 MiB threshold:
+    the flag leaves the order as it is, more than 2^24 queries (invalid ones
+    inside) give the results of the call without it bit for bit, and the
+    oracle's on a sample."""
     gen = lambda: syn.cylinder(around=128, rows=60, seed=14)
     mo, to, tl = _case(gen, lambda E: np.full(E, 5, np.int32), 4, "u8", hx.BUILD_MIPS, seed=15)
     assert tl.pool_bytes > (64 << 20)
@@ -153,6 +153,35 @@ def test_sorted_aniso_equals_unsorted_multi_chunk():
     sel = np.random.default_rng(17).choice(n, 20000, replace=False)
     _cmp(b.cpu().numpy().astype(np.float64)[sel],
          oracle.lookup_aniso(mo, to, tuple(x[sel] for x in qs), 16, nthreads=8), _tol(16, nmax=32))
+
+
+@pytest.mark.parametrize("fmt,C,n", [("f32", 4, (1 << 24) + 1237), ("f32", 2, (1 << 21) + 1), ("f32", 3, 1 << 21),
+                                     ("f16", 4, (1 << 21) + 1023), ("bf16", 3, (1 << 21) + 1025)])
+@pytest.mark.parametrize("skew", [False, True])
+def test_sorted_aniso_of_one_probe(fmt, C, n, skew):
+    """HTEX_LOOKUP_BIN with at most one probe a query sorts the 32-byte
+    queries from 2^21 on (texels of 6 bytes or more, pool above 64 MiB):
+    ragged tiles and a chunk and a part of 2^24, mixed resolutions, queries
+    all over or in two ranges only, invalid ones inside.  The unsorted call's
+    results bit for bit and the same count of invalid queries; the oracle's
+    on a sample."""
+    gen = lambda: syn.cylinder(around=128, rows=60, seed=14)
+    mo, to, tl = _case(gen, lambda E: np.where(np.arange(E) % 5 == 0, 2, 5).astype(np.int32), C, fmt,
+                       hx.BUILD_MIPS, seed=15)
+    assert tl.pool_bytes > (64 << 20) and C * hx.ELEM_SIZE[fmt] >= 6
+    qs = tuple(np.array(x) for x in _aniso_queries(mo.H, n, seed=16, lo=-8, hi=0))
+    if skew:
+        qs[0][:] = np.where(np.arange(n) % 3 == 0, 0, mo.H - 1)
+    qs[0][::70001] = -2
+    q = torch.from_numpy(hx.pack_queries_aniso(*qs)).cuda()
+    s0, s1 = (torch.zeros(1, dtype=torch.int32, device="cuda") for _ in range(2))
+    a = hx.lookup_aniso(tl, q, 1, status=s0)
+    b = hx.lookup_aniso(tl, q, 1, status=s1, flags=hx.LOOKUP_BIN)
+    assert int(s0.item()) == int(s1.item()) == int((qs[0] < 0).sum())
+    assert torch.equal(a.view(torch.int32), b.view(torch.int32))
+    sel = np.random.default_rng(17).choice(n, 20000, replace=False)
+    _cmp(b[torch.from_numpy(sel).cuda()].cpu().numpy().astype(np.float64),
+         oracle.lookup_aniso(mo, to, tuple(x[sel] for x in qs), 1, nthreads=8), _tol(1, nmax=32))
 
 
 @pytest.mark.parametrize("n", [1, 31, 33, 129, 5000])
