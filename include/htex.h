@@ -355,15 +355,16 @@ htex_status htex_lookup_host(const htex_textures* t, const htex_query* q, int64_
  *   grad_texels  device float, one per pool element (pool_bytes / element
  *                size), same element order as the pool; accumulated into
  *                (the caller zeroes it); padding elements keep their values
- *   flags        HTEX_LOOKUP_BIN: when the pool exceeds 64 MiB (and n is at least 2^18), sort the
- *                queries as htex_lookup does (chunks of 2^24, ranges of
- *                consecutive halfedges; grad_out rows move with their
- *                queries) so that the threads resident together add into
- *                a narrow range of textures; lanes of a warp whose taps
- *                coincide (the same texture, level and 2x2 block or edge
- *                texel pair) sum their contributions across the warp and
- *                one lane issues the atomics.  Scratch of 16 + 4 * channels
- *                bytes per chunk query from the library pool.
+ *   flags        HTEX_LOOKUP_BIN: when the pool exceeds 64 MiB, lanes of a
+ *                warp whose taps coincide (the same texture, level and 2x2
+ *                block or edge texel pair) sum their contributions across
+ *                the warp and one lane issues the atomics; when n is also
+ *                at least 2^20, the queries are first sorted as htex_lookup
+ *                does (chunks of 2^24, ranges of consecutive halfedges;
+ *                grad_out rows move with their queries) so that the threads
+ *                resident together add into a narrow range of textures.
+ *                The sort takes scratch of 16 + 4 * channels bytes per
+ *                chunk query from the library pool.
  *                HTEX_LOOKUP_GLOBAL ignored.
  *   d_status     as for htex_lookup
  * Uses float atomics; per three-channel texel, when grad_texels is 16-byte

@@ -460,6 +460,19 @@ constexpr int64_t kBucketTexelBytes = int64_t(32) << 20;
 // 1M: 82 / 91); the adjoint 24 / 31 / 49 and 8 / 27 / 43 us.
 constexpr int64_t kMinSortedQueries = int64_t(1) << 18;
 
+// Fewest queries the adjoint sorts under HTEX_LOOKUP_BIN.  Below, it adds up
+// what lanes of a warp share (which is what helps where many queries meet in
+// few texels) in the queries' own order.  FP32 RGBA and RGB, 0.84 to 1.1 GB,
+// us sorted / aggregated only / neither:
+//                       random halfedges                 all on one halfedge
+//               RGBA             RGB                     RGB
+//   64K     -  /  14 /  14    27 /  14 /  12             88 /   75 /   93
+//   256K    48 /  43 /  41    48 /  36 /  35            294 /  279 /  355
+//   512K    86 /  82 /  80    87 /  65 /  66            568 /  548 /  706
+//   1M     140 / 153 / 149   146 / 129 / 132           1112 / 1086 / 1406
+//   2M     237 / 301 / 290   247 / 253 / 258           2200 /   -  / 2801
+constexpr int64_t kMinSortedAdjoint = int64_t(1) << 20;
+
 // When HTEX_LOOKUP_BIN sorts anisotropic queries: of one probe each, texels
 // of 6 bytes or more, 2^21 queries or more.  Several probes spend their time
 // on lines that few queries share; sorting 32-byte queries costs more.
@@ -679,8 +692,9 @@ htex_status launch_sort_rows(const htex_textures* t, const SortPlan& P, const ht
 htex_status htex_launch_backward_sorted(const htex_textures* t, const htex_query* q, int64_t n,
                                         const float* grad_out, float* grad_texels, htex_stream stream,
                                         int32_t* d_status) {
-    if (htex_bin_shift(t) < 0 || n < kMinSortedQueries)
-        return htex_launch_backward(t, q, n, grad_out, grad_texels, 0u, stream, d_status);
+    if (htex_bin_shift(t) < 0) return htex_launch_backward(t, q, n, grad_out, grad_texels, 0u, stream, d_status);
+    if (n < kMinSortedAdjoint)
+        return htex_launch_backward(t, q, n, grad_out, grad_texels, kBackwardAggregate, stream, d_status);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const SortPlan P = sort_plan(t->H);
     const int64_t M = std::min<int64_t>(n, kSortChunk);

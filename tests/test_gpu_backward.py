@@ -108,13 +108,49 @@ def test_sorted_backward_matches_unsorted_and_oracle():
     assert int(s0.item()) == int(s1.item()) == int((h < 0).sum())
     scale = np.abs(a).max()
     assert np.abs(a - b).max() <= 1e-5 * scale
-    # oracle on the first 200k queries (the gradient is a sum over queries)
-    k = 200000
+    # oracle on the first queries, still sorted (the gradient is a sum over queries)
+    k = (1 << 20) + 3
     to = oracle.prepare_textures(mo, log2n, tex_np, 1, "f32", hx.BUILD_MIPS)
     ref = oracle.grad_to_pool_layout(to, oracle.lookup_grad(mo, to, (h[:k], u[:k], v[:k], f[:k]),
                                                             g[:k].cpu().numpy().astype(np.float64)), 4)
     c = hx.lookup_backward(tex, q[:k], g[:k], flags=hx.LOOKUP_BIN).double().cpu().numpy()
     assert np.abs(c - ref[:c.shape[0]]).max() <= 1e-5 * max(np.abs(ref).max(), 1.0)
+
+
+@pytest.mark.parametrize("C", [1, 2, 3, 4])
+@pytest.mark.parametrize("n", [1, 33, 4099, (1 << 20) - 1, 1 << 20])
+def test_binned_adjoint_below_and_at_the_sort(C, n):
+    """HTEX_LOOKUP_BIN on a pool above 64 MiB: below 2^20 queries summed over
+    the warp in their own order, from there on sorted.  Half of the queries
+    meet on one halfedge, invalid ones inside: the plain adjoint's gradient,
+    and the oracle's for the smaller batches.  Tolerance, of the largest
+    entry: 1e-5, or the rounding of up to n / 2 atomic adds into one texel in
+    two orders: each add is off by at most u = 2^-24 of a sum that grows to
+    the whole, the errors of either sign, so a third of u sqrt(n / 2) is one
+    standard deviation of a sum, and 2 u sqrt(n) more than five of the
+    difference."""
+    fs, fv, V, _ = syn.cylinder(around=128, rows=60, seed=14)
+    mesh = hx.Mesh(fs, fv, V)
+    log2n = np.full(mesh.E, 5 if C > 1 else 6, np.int32)
+    tex_np = syn.texels_f32(log2n, C, seed=15)
+    tex = hx.Textures.upload(mesh, log2n, tex_np, C, "f32", hx.BUILD_MIPS)
+    assert tex.pool_bytes > (64 << 20)
+    h, u, v, f = syn.queries(mesh.H, n, seed=16, footprint="loguniform", lo=-7, hi=0.5)
+    h[1::2] = mesh.H // 3
+    h[5::1001] = -1
+    q = torch.from_numpy(hx.pack_queries(h, u, v, f)).cuda()
+    g = torch.rand((n, C), device="cuda", generator=torch.Generator(device="cuda").manual_seed(1)) + 0.5
+    s0, s1 = (torch.zeros(1, dtype=torch.int32, device="cuda") for _ in range(2))
+    a = hx.lookup_backward(tex, q, g, status=s0)
+    b = hx.lookup_backward(tex, q, g, flags=hx.LOOKUP_BIN, status=s1)
+    assert int(s0.item()) == int(s1.item()) == int((h < 0).sum())
+    assert (a - b).abs().max() <= max(1e-5, 2 * 2.0 ** -24 * n ** 0.5) * a.abs().max()
+    if n < 5000:
+        mo = oracle.mesh_from_faces(fs, fv, V)
+        to = oracle.prepare_textures(mo, log2n, tex_np, C, "f32", hx.BUILD_MIPS)
+        ref = oracle.grad_to_pool_layout(to, oracle.lookup_grad(mo, to, (h, u, v, f), g.cpu().numpy().astype(np.float64)), 4)
+        c = b.double().cpu().numpy()
+        assert np.abs(c - ref[:c.shape[0]]).max() <= 1e-5 * np.abs(ref).max()
 
 
 @pytest.mark.parametrize("C,offsets", [(3, (0, 1, 2)), (2, (0, 2)), (1, (0, 1)), (4, (0,))])
