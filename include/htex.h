@@ -242,7 +242,7 @@ void htex_textures_destroy(htex_textures* t);
  *   q         device [n] htex_query (16-byte aligned)
  *   out       device [n][channels] float (16-byte aligned when channels = 4)
  *   flags     HTEX_LOOKUP_BIN: when the pool exceeds 64 MiB and n is at
- *             least 2^18 (below, sorting costs more than it saves),
+ *             least 2^19 (below, sorting costs more than it saves),
  *             counting-sort the queries into ranges of consecutive halfedges first, in
  *             chunks of 2^24 queries, filter them in that order and gather
  *             the results back into query order (same results, bit for bit;

@@ -454,11 +454,18 @@ constexpr int64_t kChunkBuckets = HTEX_CHUNK_BUCKETS;                // halfedge
 constexpr int64_t kBucketTexelBytes = int64_t(32) << 20;
 
 // Fewest queries HTEX_LOOKUP_BIN sorts.  Below, few queries share a texel
-// line whatever their order, and the sort's and gather's launches cost more
-// than they save: 16K / 128K / 256K random RGBA8 lookups on a 1.4 GB asset
-// take 26 / 30 / 34 us sorted, 8 / 20 / 29 us as they come (512K: 48 / 51,
-// 1M: 82 / 91); the adjoint 24 / 31 / 49 and 8 / 27 / 43 us.
-constexpr int64_t kMinSortedQueries = int64_t(1) << 18;
+// line whatever their order, and the launches of the sort and the un-sort
+// cost more than they save.  Random trilinear lookups as they come / sorted,
+// us (130k halfedges, 64x64 texels, 1.4 to 5.7 GB):
+//             256K       384K       512K        768K         1M           2M
+//   RGBA8     29 / 34    37 / 41    51 / 48     68 / 67      90 / 82    176 / 129
+//   E4M3 x4   31 / 36    39 / 42    57 / 50     76 / 71     102 / 86    199 / 140
+//   FP16 x4   37 / 37    49 / 55    70 / 64     91 / 80     122 / 94    234 / 152
+//   FP32 x4   43 / 44    55 / 64    78 / 72    100 / 92     133 / 107   253 / 173
+//   E4M3 x1   19 / 32    23 / 36    32 / 43     42 / 59      56 / 70    105 / 110
+// (one byte a texel: from 4M on, 201 / 187; at level 0 from about 2M on in
+// every format; an 81 MB pool, which L2 all but holds, never.)
+constexpr int64_t kMinSortedQueries = int64_t(1) << 19;
 
 // Fewest queries the adjoint sorts under HTEX_LOOKUP_BIN.  Below, it adds up
 // what lanes of a warp share (which is what helps where many queries meet in

@@ -280,17 +280,17 @@ def test_sorted_lookup_multi_chunk(fmt, C, n):
     _cmp(a[sel], oracle.lookup(mo, to, tuple(x[sel] for x in qs), nthreads=8))
 
 
-@pytest.mark.parametrize("n", [1, 33, 4097, 97280, 97281, 194561, (1 << 18) - 1, 1 << 18, (1 << 18) + 1])
+@pytest.mark.parametrize("n", [1, 33, 4097, 97280, 97281, 194561, 1 << 18, (1 << 19) - 1, 1 << 19, (1 << 19) + 1])
 def test_batch_sizes_give_the_same_results(n):
     """Batches below a round of every SM and below two are spread in blocks
-    of fewer warps, and HTEX_LOOKUP_BIN sorts from 2^18 queries on: the first
+    of fewer warps, and HTEX_LOOKUP_BIN sorts from 2^19 queries on: the first
     n queries of a larger batch give the same values bit for bit, plain,
     with the flag, and through the anisotropic lookup; the adjoint the same
     gradient (1e-5 of its largest entry) with and without the flag."""
     gen = lambda: syn.cylinder(around=128, rows=60, seed=14)
     mo, to, tl, *_ = _case(gen, _u(5), 4, "f32", hx.BUILD_MIPS, seed=20)
     assert tl.pool_bytes > (64 << 20)
-    h, u, v, f = syn.queries(mo.H, 300007, seed=21, footprint="loguniform")
+    h, u, v, f = syn.queries(mo.H, 600011, seed=21, footprint="loguniform")
     h[::997] = -1
     q = torch.from_numpy(hx.pack_queries(h, u, v, f)).cuda()
     ref = hx.lookup(tl, q).nan_to_num(nan=-1.0)
@@ -319,7 +319,7 @@ def test_sorted_lookup_skewed_ranges(C, skew):
     gen = lambda: syn.cylinder(around=128, rows=60, seed=14)
     mo, to, tl, *_ = _case(gen, _u(5 if C > 1 else 6), C, "u8" if C == 4 else "f32", hx.BUILD_MIPS, seed=22)
     assert tl.pool_bytes > (64 << 20)
-    n = (1 << 18) + 2049
+    n = (1 << 19) + 2049
     h, u, v, f = syn.queries(mo.H, n, seed=23, footprint="loguniform")
     if skew == "one":
         h[:] = mo.H // 2
