@@ -110,23 +110,22 @@ int htex_bin_shift(const htex_textures* t);
 
 // Resident blocks per SM of one kernel at one block size, asked of the
 // driver once per device (a property of the compiled kernel and the device;
-// the query takes longer than preparing the launch).  A kernel that needs
-// more than the default dynamic shared memory has its limit raised on the
-// same occasion.  One static object per kernel; threads may race to fill it,
-// with the same value.
+// the query takes longer than preparing the launch).  One static object per
+// kernel; threads may race to fill it, with the same value.  An answer that
+// the driver did not give is not kept.
 struct Occupancy {
     static constexpr int kDevices = 64;
     std::atomic<int> blocks[kDevices];
 
-    // 0: the shared-memory limit could not be raised
     template <class K>
     int get(K kernel, int threads, int device, size_t smem = 0) {
         const bool known = device >= 0 && device < kDevices;
         int b = known ? blocks[device].load(std::memory_order_relaxed) : 0;
         if (b > 0) return b;
-        if (smem > 0 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
-            return 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, threads, smem) != cudaSuccess || b < 1) b = 1;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, threads, smem) != cudaSuccess || b < 1) {
+            cudaGetLastError();
+            return 1;
+        }
         if (known) blocks[device].store(b, std::memory_order_relaxed);
         return b;
     }

@@ -569,10 +569,9 @@ htex_status launch_sort(const htex_textures* t, const SortPlan& P, const int4* q
                         SortRuns runs = {}) {
     constexpr int64_t TILE = ScatterSmem<QW, PC>::TILE;
     constexpr size_t smem = ScatterSmem<QW, PC>::bytes;
+    static_assert(smem <= 48 * 1024, "more dynamic shared memory than a kernel may use without asking");
     static Occupancy occupancy;
-    const int resident = occupancy.get(k_chunk_scatter<QW, PC>, kSortThreads, t->device, smem);
-    if (resident == 0) return HTEX_ERR_CUDA;
-    const int64_t blocks = int64_t(t->num_sms) * resident;
+    const int64_t blocks = int64_t(t->num_sms) * occupancy.get(k_chunk_scatter<QW, PC>, kSortThreads, t->device, smem);
     for (int64_t c0 = 0; c0 < m; c0 += kSortChunk) {
         const int64_t mc = std::min<int64_t>(kSortChunk, m - c0);
         const int64_t g = std::min<int64_t>((mc + TILE - 1) / TILE, blocks);
