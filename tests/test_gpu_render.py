@@ -154,18 +154,42 @@ def test_displacement_matches_oracle_and_is_crack_free():
                                              ("e4m3", 4, 3)])
 @pytest.mark.parametrize("T", [1, 2, 3, 8, 64])
 def test_displacement_formats_and_block_edges(dtype, C, channel, T):
-    """Mixed resolutions down to 1x1, every texel format, and the halfedges
-    per block at both ends (T = 1: 256 with a partial last block; T = 64: 1).
-    Tolerance: the FP32 lookup's 1e-5 and the position's few ulp, as above."""
+    """Mixed resolutions down to 1x1 and every texel format on a mesh so small
+    that each block takes one halfedge, of 3 points (T = 1, most of a block
+    idle) to 2145 (T = 64, several rounds).  Tolerance: the FP32 lookup's
+    1e-5 and the position's few ulp, as above."""
     fs, fv, V, pos = syn.cylinder(around=16, rows=6, seed=4)
     mo = oracle.mesh_from_faces(fs, fv, V)
     mesh = hx.Mesh(fs, fv, V)
-    assert mesh.H % 256 != 0 and mesh.H > 256
+    assert mesh.H <= 6 * torch.cuda.get_device_properties(0).multi_processor_count
     log2n = np.random.default_rng(1).integers(0, 6, mesh.E).astype(np.int32)
     flags = hx.BUILD_MIPS | hx.MIRROR_BOUNDARY
     texels = (syn.texels_u8 if dtype == "u8" else syn.texels_f32)(log2n, C, 3)
     tl = hx.Textures.upload(mesh, log2n, texels, C, dtype, flags)
     to = oracle.prepare_textures(mo, log2n, texels, C, dtype, flags)
+    got = render.Geometry(mesh, pos).displace(tl, T, 0.3, channel=channel).cpu().numpy()
+    pos32 = pos.astype(np.float32).astype(np.float64)
+    np.testing.assert_allclose(got, oracle.displace(mo, to, pos32, T, 0.3, channel=channel), atol=2e-5)
+
+
+@pytest.mark.parametrize("around,rows,T", [(40, 31, 1), (40, 31, 2), (40, 31, 3), (40, 31, 8), (100, 80, 8), (100, 80, 16),
+                                           (330, 190, 1), (330, 190, 3)])
+@pytest.mark.parametrize("dtype,C,channel", [("f32", 3, 2), ("u8", 4, 1), ("e4m3", 1, 0)])
+def test_displacement_several_halfedges_a_block(around, rows, T, dtype, C, channel):
+    """Meshes of more than six halfedges per SM, so that a block takes several
+    (as the launcher works out: few by the spread over the SMs, by the points
+    a block aims at, and the most, one per thread), the last block not full,
+    mixed resolutions.  Tolerance as above."""
+    fs, fv, V, pos = syn.cylinder(around=around, rows=rows, seed=rows)
+    mesh = hx.Mesh(fs, fv, V)
+    sms, K = torch.cuda.get_device_properties(0).multi_processor_count, (T + 1) * (T + 2) // 2
+    per_block = min(256, max(1, 2048 // K), -(-mesh.H // (6 * sms)))
+    assert per_block > 1 and mesh.H % per_block != 0 and (around < 330 or per_block > 200)
+    mo = oracle.mesh_from_faces(fs, fv, V)
+    log2n = np.random.default_rng(1).integers(0, 3, mesh.E).astype(np.int32)
+    texels = (syn.texels_u8 if dtype == "u8" else syn.texels_f32)(log2n, C, 3)
+    tl = hx.Textures.upload(mesh, log2n, texels, C, dtype, hx.BUILD_MIPS)
+    to = oracle.prepare_textures(mo, log2n, texels, C, dtype, hx.BUILD_MIPS)
     got = render.Geometry(mesh, pos).displace(tl, T, 0.3, channel=channel).cpu().numpy()
     pos32 = pos.astype(np.float32).astype(np.float64)
     np.testing.assert_allclose(got, oracle.displace(mo, to, pos32, T, 0.3, channel=channel), atol=2e-5)
