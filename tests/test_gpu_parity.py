@@ -309,6 +309,25 @@ def test_batch_sizes_give_the_same_results(n):
     assert abs(float(a.double().sum()) - 4 * valid) <= 1e-5 * 4 * max(valid, 1)
 
 
+@pytest.mark.parametrize("fmt,C", [("f16", 4), ("bf16", 4), ("f32", 2)])
+@pytest.mark.parametrize("mixed", [False, True])
+@pytest.mark.parametrize("footprint", ["zero", "loguniform"])
+def test_sorted_lookup_of_8_byte_texels(fmt, C, mixed, footprint):
+    """8-byte texels take a kernel of their own on sorted queries (every load
+    ahead of the first use): one resolution and mixed ones, level 0 and
+    trilinear, give the plain kernel's results bit for bit, and the oracle's
+    within 1e-5 on a sample."""
+    gen = lambda: syn.cylinder(around=128, rows=60, seed=14)
+    fn = (lambda E: np.where(np.arange(E) % 4 == 0, 2, 5).astype(np.int32)) if mixed else _u(5)
+    mo, to, tl, *_ = _case(gen, fn, C, fmt, hx.BUILD_MIPS | hx.MIRROR_BOUNDARY, seed=24)
+    assert tl.pool_bytes > (64 << 20)
+    qs = syn.queries(mo.H, (1 << 19) + 777, seed=25, footprint=footprint)
+    a, b = _gpu(tl, qs, flags=hx.LOOKUP_BIN), _gpu(tl, qs)
+    np.testing.assert_array_equal(a, b)
+    sel = np.random.default_rng(26).choice(len(qs[0]), 20000, replace=False)
+    _cmp(a[sel], oracle.lookup(mo, to, tuple(x[sel] for x in qs), nthreads=8))
+
+
 @pytest.mark.parametrize("C", [1, 2, 3, 4])
 @pytest.mark.parametrize("skew", ["one", "ends", "invalid", "sorted"])
 def test_sorted_lookup_skewed_ranges(C, skew):
