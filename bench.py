@@ -79,8 +79,7 @@ def run_only(args, hx, torch):
         mesh = hx.Mesh(fs, fv, V)
         log2n = np.full(mesh.E, 6, np.int32)
         tex = hx.Textures.upload(mesh, log2n, syn.texels_u8(log2n, 4, seed=21), 4, "u8", hx.BUILD_MIPS)
-        r = aniso_bench(hx, torch, stream, mesh, tex, n=args.queries, reps=args.steps, warm=args.warmup,
-                        sorted_too=False)
+        r = aniso_bench(hx, torch, stream, mesh, tex, n=args.queries, reps=args.steps, warm=args.warmup)
         print(json.dumps({"only": "aniso", **r}), flush=True)
         return
     else:
@@ -190,7 +189,7 @@ def profiled_traffic(kernel: str):
 # the files the anisotropic kernel and the adjoint are compiled from (and the build flags)
 ANISO_SOURCES = ("csrc/aniso.cu", "csrc/aniso_launch.h", "csrc/aniso_taps.h", "csrc/lookup_core.cuh", "csrc/fetch.cuh",
                  "csrc/packed.cuh", "csrc/htex_internal.h", "build.py")
-BACKWARD_SOURCES = ("csrc/backward.cu", "csrc/fetch.cuh", "csrc/htex_internal.h", "build.py")
+BACKWARD_SOURCES = ("csrc/backward.cu", "csrc/fetch.cuh", "csrc/packed.cuh", "csrc/htex_internal.h", "build.py")
 
 
 def sources_hash(rels) -> str:
@@ -880,13 +879,13 @@ def precision_asset_bench(hx, torch, stream, rows: int = 115, nq: int = 1 << 22)
     return res
 
 
-def aniso_bench(hx, torch, stream, mesh, tex, n=1 << 22, reps=10, warm=3, sorted_too=True):
+def aniso_bench(hx, torch, stream, mesh, tex, n=1 << 22, reps=10, warm=3):
     """Anisotropic lookups on the asset-scale textures: major axis
     log-uniform 2^-8..1 quad widths, anisotropy log-uniform 1..16, uniform
-    direction, at most 16 probes.  The kernel is bound by instruction issue,
-    not DRAM: its roofline entry gives the DRAM bytes per lookup and the
-    issue activity from the committed ncu summary (while the kernel's
-    sources are unchanged), the live time, and the DRAM rate they imply."""
+    direction, at most 16 probes.  The kernel is bound by random lines from
+    DRAM: its roofline entry gives the DRAM bytes per lookup and the issue
+    activity from the committed ncu summary (while the kernel's sources are
+    unchanged), the live time, and the DRAM rate they imply."""
     import htex_synth as syn
     h, u, v, _ = syn.queries(mesh.H, n, seed=31)
     rng = np.random.default_rng(32)
@@ -902,8 +901,6 @@ def aniso_bench(hx, torch, stream, mesh, tex, n=1 << 22, reps=10, warm=3, sorted
     for _ in range(warm):
         hx.lookup_aniso(tex, q, 16, out=out, stream=stream)
     ms = timed(torch, stream, lambda: hx.lookup_aniso(tex, q, 16, out=out, stream=stream), reps, warm=0)
-    sorted_ms = (timed(torch, stream, lambda: hx.lookup_aniso(tex, q, 16, out=out, stream=stream,
-                                                              flags=hx.LOOKUP_BIN), reps) if sorted_too else None)
     prof = profiled_values("lookup_aniso.md", ANISO_SOURCES)
     peak, _ = hbm_peak()
     roof = {"bound": "random DRAM lines", "unit": "GB/s", "peak": peak}
@@ -914,7 +911,6 @@ def aniso_bench(hx, torch, stream, mesh, tex, n=1 << 22, reps=10, warm=3, sorted
                      "source": "profiles/lookup_aniso.md (ncu, quarter-size asset)"})
     return {"queries": n, "max_aniso": 16, "mean_probes": float(k.mean()), "ms": ms,
             "lookups_per_s": n / (ms / 1e3), "probes_per_s": float(k.sum()) / (ms / 1e3),
-            "sorted_ms": sorted_ms, "sorted_lookups_per_s": n / (sorted_ms / 1e3) if sorted_ms else None,
             "roofline": roof}
 
 
