@@ -243,9 +243,10 @@ void htex_textures_destroy(htex_textures* t);
  *   out       device [n][channels] float (16-byte aligned when channels = 4)
  *   flags     HTEX_LOOKUP_BIN: when the pool exceeds 64 MiB and n is at
  *             least 2^19 (below, sorting costs more than it saves),
- *             counting-sort the queries into ranges of consecutive halfedges first, in
- *             chunks of 2^24 queries, filter them in that order and gather
- *             the results back into query order (same results, bit for bit;
+ *             counting-sort the queries into ranges of consecutive
+ *             halfedges first, in chunks of 2^24 queries, filter them in
+ *             that order and put the results back into query order (same
+ *             results, bit for bit;
  *             scratch of about 19 + 4 * channels bytes per chunk query,
  *             allocated stream-ordered on 'stream' from a library-owned
  *             pool and released there; HTEX_ERR_OUT_OF_MEMORY when it cannot
@@ -295,7 +296,10 @@ htex_status htex_lookup_aniso(const htex_textures* t, const htex_query_aniso* q,
 
 /* The two halves of HTEX_LOOKUP_BIN as calls of their own, for callers
  * that filter one sorted batch more than once (several texture sets on
- * one mesh) or time the filter on its own.  The paper has no counterpart:
+ * one mesh) or time the filter on its own; for one lookup the flag is
+ * faster (16M RGBA8 lookups 809 us against 847 in three calls, 4M FP32 RG
+ * 223 against 266), since that call knows that its queries are sorted and
+ * puts the results back in whole runs.  The paper has no counterpart:
  * query order does not change any result (each query is filtered on its
  * own, Section 4.4, Alg. 3), only which texels share L2 at a time.
  *

@@ -94,9 +94,10 @@ constexpr int kStagedThreads = 1024;
 
 // SORTED: the queries come sorted by halfedge range.  Their texels then
 // mostly come from L1 and L2, and 8-byte texels too are worth loading ahead
-// in two registers each: 4M sorted FP16 RGBA / FP32 RG lookups 255 / 235 ->
-// 227 / 192 us; in a random order 203 -> 212 and 83 -> 85 us (2M, 1M), so
-// not there.  Other texel sizes: the same kernel either way.
+// in two registers each: 4M sorted FP16 RGBA / FP32 RG lookups, the whole
+// call, 279 / 259 -> 262 / 218 us on 130k halfedges (2.9 GB), 246 / 228 ->
+// 219 / 182 us on 104k (0.56 GB); in a random order 203 -> 212 and 83 -> 85
+// us (2M, 1M), so not there.  Other texel sizes: the same kernel either way.
 template <int DT, int C, bool BINNED, bool UNI, bool SORTED>
 __global__ void __launch_bounds__(kGlobalThreads, HTEX_GLOBAL_MIN_BLOCKS) k_lookup_global(Asset<GlobalSpace> A, FwdParams p) {
     constexpr bool DEFER = Raw<DT, C>::PACKED || (SORTED && Raw<DT, C>::DOUBLE);

@@ -12,16 +12,16 @@
 // halfedge) is kept per pixel with atomicMin, so ties go to the smaller
 // halfedge id.  A resolve pass turns each pixel's key into a query from the
 // projected triangle, which the first pass left in scratch or (meshes fine
-// beside the frame) is projected again: barycentrics at the
-// pixel centre corrected for perspective, and the footprint max(|d(u,v)/dx|,
-// |d(u,v)/dy|) from the same triangle's barycentrics one pixel right and one
-// pixel down.  Triangles with a vertex behind the camera (w <= 0) are not
-// drawn.
+// beside the frame) is projected again: barycentrics at the pixel centre
+// corrected for perspective, and the footprint max(|d(u,v)/dx|, |d(u,v)/dy|)
+// from the same triangle's barycentrics one pixel right and one pixel down.
+// Triangles with a vertex behind the camera (w <= 0) are not drawn.
 //
 // Bound by instruction issue.  522,370 halfedges at 1920x1080 (a thread a
 // triangle, then the projection again per pixel: 52 and 38 us): covering
-// 45 us, resolving 23 us; the covering with 5 blocks per SM (4 or 6: 3% of
-// the frame slower; one block per 256 triangles, smaller blocks: within 1%).
+// 45 us, resolving 23 us; the covering with 5 blocks per SM (48 registers and
+// 24 bytes of spills; 4 or 6: 3% of the frame slower; one block per 256
+// triangles, smaller blocks: within 1%).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
