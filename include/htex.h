@@ -246,12 +246,12 @@ void htex_textures_destroy(htex_textures* t);
  *             counting-sort the queries into ranges of consecutive
  *             halfedges first, in chunks of 2^24 queries, filter them in
  *             that order and put the results back into query order (same
- *             results, bit for bit;
- *             scratch of about 19 + 4 * channels bytes per chunk query,
- *             allocated stream-ordered on 'stream' from a library-owned
- *             pool and released there; HTEX_ERR_OUT_OF_MEMORY when it cannot
- *             be had); HTEX_LOOKUP_GLOBAL: never stage the pool in shared
- *             memory (by default a pool of at most 96 KiB is staged)
+ *             results, bit for bit; scratch of about 19 + 4 * channels
+ *             bytes per chunk query, allocated stream-ordered on 'stream'
+ *             from a library-owned pool and released there;
+ *             HTEX_ERR_OUT_OF_MEMORY when it cannot be had);
+ *             HTEX_LOOKUP_GLOBAL: never stage the pool in shared memory
+ *             (by default a pool of at most 96 KiB is staged)
  *   d_status  device int32, nullable: incremented once per invalid query
  * For each query: own = quad of Edge(h) at Alg. 2 (h, (u, v)), then the
  * quads of Next(h) at (v, -u) and of Prev(h) at (-v, u); each fetch is a
@@ -282,8 +282,8 @@ htex_status htex_lookup(const htex_textures* t, const htex_query* q, int64_t n, 
  *   flags      HTEX_LOOKUP_BIN: with max_aniso = 1, texels of 6 bytes or
  *              more, 2^21 queries or more and a pool above 64 MiB, sort the
  *              queries as htex_lookup does (scratch of about 35 + 4 *
- *              channels bytes per chunk query); else they are filtered in
- *              their given order, which is faster.  The same results
+ *              channels bytes per chunk query, while it can be had); else
+ *              they are filtered in their given order.  The same results
  *              either way, bit for bit: each query's probes are summed in
  *              an order of its own
  *   out        device [n][channels] float (alignment as htex_lookup)

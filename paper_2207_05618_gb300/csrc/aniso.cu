@@ -413,6 +413,9 @@ extern "C" htex_status htex_lookup_aniso(const htex_textures* t, const htex_quer
     if ((reinterpret_cast<uintptr_t>(q) & 15u) != 0) return HTEX_ERR_INVALID_ARG;
     const uintptr_t out_align = t->C == 4 ? 16u : (t->C == 2 ? 8u : 4u);
     if ((reinterpret_cast<uintptr_t>(out) & (out_align - 1)) != 0) return HTEX_ERR_INVALID_ARG;
-    if (flags & HTEX_LOOKUP_BIN) return htex_launch_aniso_sorted(t, q, n, max_aniso, out, stream, d_status);
+    if (flags & HTEX_LOOKUP_BIN) {
+        const htex_status st = htex_launch_aniso_sorted(t, q, n, max_aniso, out, stream, d_status);
+        if (st != HTEX_ERR_OUT_OF_MEMORY) return st;   // no memory to sort in (nothing launched): in the given order
+    }
     return htex_launch_aniso(t, q, n, max_aniso, out, stream, d_status);
 }
