@@ -343,7 +343,7 @@ __global__ void k_resolve(htex_geometry g, Camera cam, const unsigned long long*
         // 16 bytes a store (the entry point checks the alignment): word by word
         // every store of a warp touches all of its lines.  2 megapixels of 57k
         // halfedges, the whole call: anisotropic queries 101 -> 70 us, 8
-        // megapixels 344 -> 224
+        // megapixels 343 -> 233
         float4* const to = reinterpret_cast<float4*>(q + i);
         if constexpr (std::is_same<Q, htex_query>::value) {
             to[0] = make_float4(__int_as_float(h), u, vv, d[0]);
@@ -493,15 +493,13 @@ htex_status rasterize(const htex_geometry* g, const float* view_proj, int32_t wi
     // 45, 2.2: 129 / 127; 14,400 pixels of 57k halfedges 14.4 / 16.4.
     const size_t vis_b = (size_t(n) * 8 + 63) & ~size_t(63);
     void* vis = nullptr;
-    bool kept = g->H <= std::max<int64_t>(n, int64_t(1) << 18);
-    kept = kept && cudaMallocFromPoolAsync(&vis, vis_b + size_t(g->H) * 64, pool, s) == cudaSuccess;
-    if (!kept) {
+    const auto allocate = [&](size_t bytes) {
+        if (cudaMallocFromPoolAsync(&vis, bytes, pool, s) == cudaSuccess) return true;
         cudaGetLastError();
-        if (cudaMallocFromPoolAsync(&vis, vis_b, pool, s) != cudaSuccess) {
-            cudaGetLastError();
-            return HTEX_ERR_OUT_OF_MEMORY;
-        }
-    }
+        return false;
+    };
+    const bool kept = g->H <= std::max<int64_t>(n, int64_t(1) << 18) && allocate(vis_b + size_t(g->H) * 64);
+    if (!kept && !allocate(vis_b)) return HTEX_ERR_OUT_OF_MEMORY;
     auto* v = static_cast<unsigned long long*>(vis);
     auto* screens = kept ? reinterpret_cast<float4*>(static_cast<uint8_t*>(vis) + vis_b) : nullptr;
     k_clear<<<grid_for(int64_t(vis_b / 16)), kThreads, 0, s>>>(static_cast<ulonglong2*>(vis), int64_t(vis_b / 16));
